@@ -326,7 +326,10 @@ int run_adjoint(grav_plan* p, const void* r, void* grad, void* wa, void* wb, int
     ColumnArgs a{p->ny, p->ny_pad, p->nz, p->ncomp, p->kx_count, p->jp, p->imag_mask, p->oddv_mask,
                  p->log_t - (p->log_py - 1), p->log_t - p->log_py};
     // FP32 2048 x 2048 plans: tile-major column output, read back by whole tiles
-    if constexpr (sizeof(R) == 4) a.z_tiled = adjoint_tiled_ok(p->log_py - 1, p->log_px, p->nx, a) ? 1 : 0;
+    if constexpr (sizeof(R) == 4) {
+        a.z_tiled = adjoint_tiled_ok(p->log_py - 1, p->log_px, p->nx, a) ? 1 : 0;
+        a.z_summed = adjoint_summed(p->log_py - 1) ? 1 : 0;
+    }
     if (spec_of) {
         a.spec_count = batch;
         for (int i = 0; i < batch; ++i) a.spec_of[i] = spec_of[i];
@@ -341,7 +344,8 @@ int run_adjoint(grav_plan* p, const void* r, void* grad, void* wa, void* wb, int
                                  (size_t)p->nx, p->nx, p->tw, p->log_t, s,
                                  Batch{batch, cs, (size_t)p->nz * p->ny * p->nx}, p->err_flag);
     } else {
-        e = launch_row_c2r<R>(p->log_px, wa, (const unsigned char*)wa + half, p->ny, p->nz, p->ny_pad, (R*)grad,
+        const void* wa1 = a.z_summed ? nullptr : (const unsigned char*)wa + half;
+        e = launch_row_c2r<R>(p->log_px, wa, wa1, p->ny, p->nz, p->ny_pad, (R*)grad,
                               (size_t)p->nx, p->nx, p->tw, p->log_t, s,
                               Batch{batch, cs, (size_t)p->nz * p->ny * p->nx});
     }

@@ -510,29 +510,39 @@ cudaError_t r2c_impl(const R* in, size_t in_ostride, size_t in_istride, int l_in
             return cudaGetLastError();
         }
     }
-    // float rows of at most P/2 values, whole 16-byte vectors, aligned
-    if constexpr (sizeof(R) == 4) {
+    if constexpr (sizeof(R) == 4 && LOGP >= 7 && LOGP <= 11) {
+        // register transforms by groups of lanes (row_groups.cu); every plan's
+        // rows and workspaces satisfy its conditions
+        return launch_row_r2c_group(LOGP, in, in_ostride, in_istride, l_in, I, O, out, i_pad, tw, log_t, s, b);
+    } else if constexpr (sizeof(R) == 4) {
+        // float rows of at most P/2 values, whole 8-byte pairs, aligned
         const bool vec = l_in <= (1 << LOGP) / 2 && l_in % 2 == 0 && in_istride % 2 == 0 && in_ostride % 2 == 0 &&
                          b.in % 2 == 0 && (reinterpret_cast<uintptr_t>(in) & 7) == 0 && i_pad % 2 == 0;
         if (vec) return r2c_launch<R, LOGP, true>(in, in_ostride, in_istride, l_in, I, O, out, i_pad, tw, log_t, s, b);
+        return r2c_launch<R, LOGP, false>(in, in_ostride, in_istride, l_in, I, O, out, i_pad, tw, log_t, s, b);
+    } else {
+        return r2c_launch<R, LOGP, false>(in, in_ostride, in_istride, l_in, I, O, out, i_pad, tw, log_t, s, b);
     }
-    return r2c_launch<R, LOGP, false>(in, in_ostride, in_istride, l_in, I, O, out, i_pad, tw, log_t, s, b);
 }
 
 template <typename R, int LOGP>
 cudaError_t c2r_impl(const void* in0, const void* in1, int I, int O, int i_pad, R* out, size_t out_stride, int l_out,
                      const void* tw, int log_t, cudaStream_t s, Batch b) {
-    using C = typename cplx<R>::type;
-    constexpr int NSEQ = nseq_for<R>(LOGP);
-    constexpr int NT = 512;
-    const size_t smem = (size_t)NSEQ * seq_stride<C>(1 << LOGP) * sizeof(C);
-    constexpr auto k = row_c2r_kernel<R, LOGP, NSEQ, NT>;
-    cudaError_t e = ensure_smem_limit<k>();
-    if (e != cudaSuccess) return e;
-    dim3 grid((I + 2 * NSEQ - 1) / (2 * NSEQ), O, b.count);
-    k<<<grid, NT, smem, s>>>((const C*)in0, (const C*)in1, I, O, i_pad, out, out_stride, l_out, (const C*)tw,
-                             log_t - LOGP, b.in, b.out);
-    return cudaGetLastError();
+    if constexpr (sizeof(R) == 4 && LOGP >= 7 && LOGP <= 11) {
+        return launch_row_c2r_group(LOGP, in0, in1, I, O, i_pad, out, out_stride, l_out, tw, log_t, s, b);
+    } else {
+        using C = typename cplx<R>::type;
+        constexpr int NSEQ = nseq_for<R>(LOGP);
+        constexpr int NT = 512;
+        const size_t smem = (size_t)NSEQ * seq_stride<C>(1 << LOGP) * sizeof(C);
+        constexpr auto k = row_c2r_kernel<R, LOGP, NSEQ, NT>;
+        cudaError_t e = ensure_smem_limit<k>();
+        if (e != cudaSuccess) return e;
+        dim3 grid((I + 2 * NSEQ - 1) / (2 * NSEQ), O, b.count);
+        k<<<grid, NT, smem, s>>>((const C*)in0, (const C*)in1, I, O, i_pad, out, out_stride, l_out, (const C*)tw,
+                                 log_t - LOGP, b.in, b.out);
+        return cudaGetLastError();
+    }
 }
 
 }  // namespace

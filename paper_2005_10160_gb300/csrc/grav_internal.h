@@ -55,6 +55,8 @@ struct ColumnArgs {
                          // 1 = Z[r][n][y / 8][kx][8], row pair (y % 8) / 2 at 16-byte position
                          // ((y % 8) / 2 + kx / 2) % 4 of the run (ny_pad a multiple of 8;
                          // see launch_row_c2r_tiled)
+    int z_summed;        // adjoint output Z[kx][n][y] holds the sum of both ky parities (untiled;
+                         // see adjoint_summed)
     // Batched calls across plans of equal sizes and components: request b
     // reads the kernel spectra at spec_of[b] (spec_count > 0); with
     // spec_count == 0 every request reads the kernel's spec argument.
@@ -129,6 +131,32 @@ inline cudaError_t ensure_smem_limit() {
     return e;
 }
 
+// Launch of a kernel whose predecessor on the stream may still be running:
+// its CTAs may start once every CTA of the predecessor has called
+// chain_trigger() or ended.  The kernel calls chain_wait() before it reads or
+// writes anything another kernel of the stream touches (what a plan holds for
+// good, the spectra and twiddles, may be read ahead of it), and reads the
+// predecessor's output past L1 (__ldcg).
+template <typename... P, typename... A>
+inline cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t s,
+                                  A... args) {
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+#ifdef __CUDACC__
+__device__ __forceinline__ void chain_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+#endif
+
 // Per-request strides of a batched call (elements of the buffer's own type);
 // unused when batch == 1.
 struct Batch {
@@ -182,6 +210,16 @@ cudaError_t launch_row_c2r(int log_p, const void* in0, const void* in1, int I, i
                            R* out, size_t out_stride, int l_out, const void* tw, int log_t,
                            cudaStream_t s, Batch b = Batch());
 
+// FP32 rows of P = 2^log_p = 128 .. 2048 points with at most P / 2 nonzero
+// inputs or wanted outputs (row_groups.cu): arguments and layouts as the
+// launchers above; cudaErrorNotSupported when the sizes or alignments do not
+// fit (other lengths, l_in or l_out > P / 2, odd i_pad or batch stride, a
+// workspace that is not 16-byte aligned), and the caller takes another kernel.
+cudaError_t launch_row_r2c_group(int log_p, const float* in, size_t in_ostride, size_t in_istride, int l_in, int I,
+                                 int O, void* out, int i_pad, const void* tw, int log_t, cudaStream_t s, Batch b);
+cudaError_t launch_row_c2r_group(int log_p, const void* in0, const void* in1, int I, int O, int i_pad, float* out,
+                                 size_t out_stride, int l_out, const void* tw, int log_t, cudaStream_t s, Batch b);
+
 // Forward column stage for 512-point FP32 columns (Py = 1024) with both ky
 // parities of a column in one CTA and two transforms per warp
 // (col_fwd512_f32.cu).  Same arguments and layouts as the column launchers
@@ -194,6 +232,17 @@ cudaError_t launch_forward_wf512(const ColumnArgs& a, const void* X, const float
 // err is null or a.z_tiled is set.
 cudaError_t launch_adjoint_wf512(const ColumnArgs& a, const void* Xr, const float* spec, void* Z, const void* tw,
                                  int* err, cudaStream_t s, Batch b);
+
+// Column stages for 64-, 128- and 256-point FP32 columns (33 <= ny <= 256;
+// col_groups.cuh).  Same layouts as the column launchers below, but the
+// adjoint writes the summed column output (ColumnArgs::z_summed).
+cudaError_t launch_forward_groups(int log_n, const ColumnArgs& a, const void* X, const float* spec, void* Y,
+                                  const void* tw, cudaStream_t s, Batch b);
+cudaError_t launch_adjoint_groups(int log_n, const ColumnArgs& a, const void* Xr, const float* spec, void* Z,
+                                  const void* tw, cudaStream_t s, Batch b);
+// Whether the FP32 adjoint column stage of 2^log_n-point columns adds the two
+// ky parities itself and writes Z[kx][n][y].
+constexpr bool adjoint_summed(int log_n) { return log_n >= 6 && log_n <= 8; }
 
 // Adjoint inverse rows from the tiled column output (ColumnArgs::z_tiled):
 // in_r[n][y / 8][kx][8] (swizzled as described there) for r = 0, 1 (in1 = in0 + one half), summed, kx

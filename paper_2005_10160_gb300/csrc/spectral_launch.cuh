@@ -42,14 +42,19 @@ cudaError_t forward_impl(const ColumnArgs& a, const void* X, const R* spec, void
             return cudaGetLastError();
         }
     }
-    const FwdSmem L = forward_smem<R>(LOGN, a.ny_pad, a.ncomp, a.jp, kMaxSmemOptin);
-    if (L.depth == 0) return cudaErrorInvalidConfiguration;
-    constexpr auto k = forward_column_kernel<R, LOGN, NC>;
-    cudaError_t e = ensure_smem_limit<k>();
-    if (e != cudaSuccess) return e;
-    k<<<dim3(2 * a.kx_count, b.count), ColShape<LOGN>::J, L.total, s>>>(a, L, (const C*)X, spec, (C*)Y, (const C*)tw,
-                                                                         err, b.in, b.out);
-    return cudaGetLastError();
+    if constexpr (sizeof(R) == 4 && LOGN >= 6 && LOGN <= 8) {
+        // 64- to 256-point FP32 columns: lane-group transforms, eight layers a round
+        return launch_forward_groups(LOGN, a, X, (const float*)spec, Y, tw, s, b);
+    } else {
+        const FwdSmem L = forward_smem<R>(LOGN, a.ny_pad, a.ncomp, a.jp, kMaxSmemOptin);
+        if (L.depth == 0) return cudaErrorInvalidConfiguration;
+        constexpr auto k = forward_column_kernel<R, LOGN, NC>;
+        cudaError_t e = ensure_smem_limit<k>();
+        if (e != cudaSuccess) return e;
+        k<<<dim3(2 * a.kx_count, b.count), ColShape<LOGN>::J, L.total, s>>>(a, L, (const C*)X, spec, (C*)Y,
+                                                                             (const C*)tw, err, b.in, b.out);
+        return cudaGetLastError();
+    }
 }
 
 #define GRAV_NC_SWITCH(R, L)                                                     \
@@ -133,13 +138,18 @@ cudaError_t adjoint_impl(const ColumnArgs& a, const void* Xr, const R* spec, voi
         const cudaError_t e = launch_adjoint_wf512(a, Xr, (const float*)spec, Z, tw, err, s, b);
         if (e != cudaErrorNotSupported) return e;
     }
-    constexpr auto k = adjoint_column_kernel<R, LOGN, CPG>;
-    const size_t smem = column_smem_bytes<R>(LOGN);
-    cudaError_t e = ensure_smem_limit<k>();
-    if (e != cudaSuccess) return e;
-    k<<<dim3(a.kx_count, 2, b.count), ColShape<LOGN>::NT, smem, s>>>(a, (const C*)Xr, spec, (C*)Z, (const C*)tw, b.in,
-                                                                       b.out);
-    return cudaGetLastError();
+    if constexpr (sizeof(R) == 4 && LOGN >= 6 && LOGN <= 8) {
+        static_assert(adjoint_summed(LOGN), "these kernels write the summed column output");
+        return launch_adjoint_groups(LOGN, a, Xr, (const float*)spec, Z, tw, s, b);
+    } else {
+        constexpr auto k = adjoint_column_kernel<R, LOGN, CPG>;
+        const size_t smem = column_smem_bytes<R>(LOGN);
+        cudaError_t e = ensure_smem_limit<k>();
+        if (e != cudaSuccess) return e;
+        k<<<dim3(a.kx_count, 2, b.count), ColShape<LOGN>::NT, smem, s>>>(a, (const C*)Xr, spec, (C*)Z, (const C*)tw,
+                                                                           b.in, b.out);
+        return cudaGetLastError();
+    }
 }
 
 #define GRAV_CPG_SWITCH(FN, R, L, ...)                       \
