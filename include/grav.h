@@ -165,6 +165,31 @@ int grav_forward_batch_plans(int batch, grav_plan* const* plans, const void* rho
 int grav_adjoint_batch_plans(int batch, grav_plan* const* plans, const void* r_dev, void* grad_dev,
                              void* workspace_dev, void* stream);
 
+/* Damped CGLS (least-squares inversion, Sec. 1 and Sec. 4) with depth weights,
+ * enqueued whole on a stream: minimises ||W (G m - d)||^2 + lam ||W_m m||^2 by
+ * conjugate gradients on the normal equations in x = W_m m from x = 0, one
+ * forward and one adjoint per step.  All scalars stay on the device: nothing
+ * waits for the host.  When (s, s) is exactly 0 the remaining steps change
+ * nothing.
+ *   d_dev           device [ncomp][ny][nx] data
+ *   w_dev           device [ncomp][ny][nx] data weights (1 / sigma)
+ *   wm_dev          device [nz] depth weights of the layers
+ *   iters           steps (>= 0), the same value in both calls
+ *   keep_models     0: models_dev is device [nz][ny][nx] and receives the model
+ *                   m = x / w_n after the last step (0 without steps);
+ *                   1: [iters][nz][ny][nx], the model after every step.
+ *                   16-byte aligned
+ *   objectives_dev  device double [iters + 1]: the objective after 0, 1, ... steps
+ *   work_dev        device scratch of grav_cgls_work_bytes(plan, iters) bytes,
+ *                   256-byte aligned, kept from start to steps
+ * Element types as grav_forward.  Both calls use the plan's workspaces.
+ * Return GRAV_OK, GRAV_EINVAL or GRAV_ECUDA. */
+size_t grav_cgls_work_bytes(const grav_plan* plan, int iters);
+int grav_cgls_start(grav_plan* plan, const void* d_dev, const void* w_dev, const void* wm_dev, int iters,
+                    void* work_dev, void* stream);
+int grav_cgls_steps(grav_plan* plan, const void* w_dev, const void* wm_dev, double lam, int iters, int keep_models,
+                    void* models_dev, double* objectives_dev, void* work_dev, void* stream);
+
 /* Release the plan and its device memory (waits for the device first).
  * NULL is ignored. */
 void grav_plan_destroy(grav_plan* plan);

@@ -48,6 +48,9 @@ EXPORTED = (
     "grav_adjoint3d",
     "grav_forward_batch_plans",
     "grav_adjoint_batch_plans",
+    "grav_cgls_work_bytes",
+    "grav_cgls_start",
+    "grav_cgls_steps",
 )
 
 
@@ -124,6 +127,12 @@ def lib() -> ctypes.CDLL:
             L.grav_forward3d.restype = i
             L.grav_adjoint3d.argtypes = [p, p, p, p]
             L.grav_adjoint3d.restype = i
+            L.grav_cgls_work_bytes.argtypes = [p, i]
+            L.grav_cgls_work_bytes.restype = sz
+            L.grav_cgls_start.argtypes = [p, p, p, p, i, p, p]
+            L.grav_cgls_start.restype = i
+            L.grav_cgls_steps.argtypes = [p, p, p, d, i, i, p, p, p, p]
+            L.grav_cgls_steps.restype = i
             _lib = L
     return _lib
 
@@ -262,3 +271,16 @@ def grav_forward_batch_plans(plans, rho_ptr, out_ptr, ws_ptr, stream=0) -> int:
 def grav_adjoint_batch_plans(plans, r_ptr, grad_ptr, ws_ptr, stream=0) -> int:
     return _check(lib().grav_adjoint_batch_plans(len(plans), _plan_array(plans), r_ptr, grad_ptr, ws_ptr or None,
                                                  stream or None))
+
+
+def grav_cgls_work_bytes(plan, iters) -> int:
+    return int(lib().grav_cgls_work_bytes(plan, int(iters)))
+
+
+def grav_cgls_start(plan, d_ptr, w_ptr, wm_ptr, iters, work_ptr, stream=0) -> int:
+    return _check(lib().grav_cgls_start(plan, d_ptr, w_ptr, wm_ptr, int(iters), work_ptr, stream or None))
+
+
+def grav_cgls_steps(plan, w_ptr, wm_ptr, lam, iters, keep_models, models_ptr, objectives_ptr, work_ptr, stream=0) -> int:
+    return _check(lib().grav_cgls_steps(plan, w_ptr, wm_ptr, float(lam), int(iters), 1 if keep_models else 0,
+                                        models_ptr or None, objectives_ptr, work_ptr, stream or None))

@@ -1,0 +1,414 @@
+// The damped CGLS loop (least-squares density inversion, Sec. 1 and Sec. 4)
+// enqueued whole on one stream: forward and adjoint products plus the vector
+// updates between them, with every scalar of the recurrence on the device, so
+// the host neither waits nor launches per dot product.
+//
+// In x = W_m m with s = A^T r - lam x, A = W_d G W_m^-1:
+//   q = A p;  alpha = (s, s) / ((q, q) + lam (p, p));  x += alpha p;  r -= alpha q
+//   s' = A^T r - lam x;  beta = (s', s') / (s, s);  p = s' + beta p
+// The model-size vectors are touched twice per iteration:
+//   step_model   x += alpha p, s = g / w_n - lam x (in place of g = G^T w r), (s, s), (x, x)
+//   next_dir     p = s + beta p, t = p / w_n (the next forward's input), (p, p)
+// i.e. nine passes over a vector in all, where separate operations took
+// about forty.  A dot product is one FP64 partial per block; the last block to
+// finish adds them in a fixed order, so the kernels that use it read one number.
+//
+// 512 x 512 x 64, two components: 0.57 GB per iteration in 0.15 ms (step_model
+// 68 us, next_dir 55, the three data-size kernels 10 each); three iterations
+// from 4.68 to 2.30 ms, 1.9 ms of vector operations before.
+//
+// FP64 instructions run at 1/64 of the FP32 rate here, and two products and
+// two widenings per element in FP64 took longer than the memory traffic
+// (step_model 174 us at 512 x 512 x 64 for 0.34 GB).  A thread therefore keeps
+// an FP32 plan's sum as an unevaluated pair of floats: the product's rounding
+// error by fused multiply-add, the sum's by the two-sum of Knuth (TAOCP 2,
+// 4.2.2), both added to the low part; products are exact and the sum is good
+// to about 2^-45, more than the separately rounded FP32 products had before.
+#include <algorithm>
+
+#include "grav_internal.h"
+
+namespace grav {
+
+namespace {
+
+constexpr int kVecThreads = 256;
+constexpr int kMaxParts = 1216;  // most blocks (partial sums) of a vector kernel: 8 per SM
+
+// Sum over the block, valid in thread 0.
+__device__ __forceinline__ double block_sum(double v) {
+    __shared__ double part[kVecThreads / 32];
+    __syncthreads();  // an earlier sum's values are read
+    for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = v;
+    __syncthreads();
+    double s = 0.0;
+    if (threadIdx.x == 0)
+        for (int w = 0; w < kVecThreads / 32; ++w) s += part[w];
+    return s;
+}
+
+// A dot product in the making: one partial per block, the number of blocks
+// done (0 before and after each use), and the result.
+struct Dot {
+    double value;
+    unsigned done, pad;
+    double parts[kMaxParts];
+};
+
+// Every block of the grid hands in its share (all threads call this); the last
+// one adds the partials up in block order.
+__device__ __forceinline__ void put_dot(Dot* d, double share) {
+    __shared__ bool last;
+    const unsigned nb = gridDim.x * gridDim.y, b = blockIdx.y * gridDim.x + blockIdx.x;
+    const double s = block_sum(share);
+    if (threadIdx.x == 0) {
+        d->parts[b] = s;
+        __threadfence();
+        last = atomicInc(&d->done, nb - 1) == nb - 1;  // wraps to 0 for the next use
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    double v = 0.0;
+    for (unsigned i = threadIdx.x; i < nb; i += kVecThreads) v += __ldcg(&d->parts[i]);
+    v = block_sum(v);
+    if (threadIdx.x == 0) d->value = v;
+}
+
+// Sum of squares of one thread's values.
+template <typename R> struct Squares;
+template <> struct Squares<double> {
+    double s = 0.0;
+    __device__ __forceinline__ void add(double v) { s += v * v; }
+    __device__ __forceinline__ double get() const { return s; }
+};
+template <> struct Squares<float> {
+    float hi = 0.f, lo = 0.f;
+    __device__ __forceinline__ void add(float v) {
+        const float p = __fmul_rn(v, v), pe = __fmaf_rn(v, v, -p);
+        const float t = __fadd_rn(hi, p), z = __fsub_rn(t, hi);
+        const float te = __fadd_rn(__fsub_rn(hi, __fsub_rn(t, z)), __fsub_rn(p, z));
+        hi = t;
+        lo = __fadd_rn(lo, __fadd_rn(pe, te));
+    }
+    __device__ __forceinline__ double get() const {
+        // past the FP32 range the corrections are not numbers; the sum is
+        return isfinite(lo) ? (double)hi + (double)lo : (double)hi;
+    }
+};
+
+template <typename R, int VEC> struct alignas(sizeof(R) * VEC) Pack { R v[VEC]; };
+
+// (s, s) before the step, (p, p), (q, q)
+struct Scalars {
+    const Dot *gamma, *pp, *qq;
+    double lam;
+};
+// alpha, the same value in every thread.  A vanished gradient ends the
+// recurrence: nothing moves any more.
+__device__ __forceinline__ double step_length(const Scalars& k) {
+    __shared__ double alpha;
+    if (threadIdx.x == 0) {
+        const double gamma = k.gamma->value;
+        alpha = gamma == 0.0 ? 0.0 : gamma / (k.qq->value + k.lam * k.pp->value);
+    }
+    __syncthreads();
+    return alpha;
+}
+
+// r = w d, wr = w r, (r, r)
+template <typename R>
+__global__ void __launch_bounds__(kVecThreads) cgls_first_data(const R* __restrict__ d, const R* __restrict__ w, R* __restrict__ r,
+                                                               R* __restrict__ wr, size_t n, Dot* rr) {
+    Squares<R> s;
+    for (size_t i = (size_t)blockIdx.x * kVecThreads + threadIdx.x; i < n; i += (size_t)gridDim.x * kVecThreads) {
+        const R v = w[i] * d[i];
+        r[i] = v;
+        wr[i] = w[i] * v;
+        s.add(v);
+    }
+    put_dot(rr, s.get());
+}
+
+// q = w y in place, (q, q)
+template <typename R>
+__global__ void __launch_bounds__(kVecThreads) cgls_weigh(const R* __restrict__ w, R* __restrict__ q, size_t n, Dot* qq) {
+    Squares<R> s;
+    for (size_t i = (size_t)blockIdx.x * kVecThreads + threadIdx.x; i < n; i += (size_t)gridDim.x * kVecThreads) {
+        const R v = w[i] * q[i];
+        q[i] = v;
+        s.add(v);
+    }
+    put_dot(qq, s.get());
+}
+
+// r -= alpha q, wr = w r, (r, r)
+template <typename R>
+__global__ void __launch_bounds__(kVecThreads) cgls_step_data(Scalars k, const R* __restrict__ w, const R* __restrict__ q, R* __restrict__ r,
+                                                              R* __restrict__ wr, size_t n, Dot* rr) {
+    const R alpha = (R)step_length(k);
+    Squares<R> s;
+    for (size_t i = (size_t)blockIdx.x * kVecThreads + threadIdx.x; i < n; i += (size_t)gridDim.x * kVecThreads) {
+        const R v = r[i] - alpha * q[i];
+        r[i] = v;
+        wr[i] = w[i] * v;
+        s.add(v);
+    }
+    put_dot(rr, s.get());
+}
+
+// Model-size kernels: block rows take layers blockIdx.y, blockIdx.y + gridDim.y,
+// ..., so that the depth weight is constant over a block's inner loop.
+#define GRAV_FOR_LAYERS                                        \
+    for (int n = blockIdx.y; n < nz; n += gridDim.y) {         \
+        const R wn = wm[n];                                    \
+        const size_t base = (size_t)n * plane;                 \
+        for (size_t i = ((size_t)blockIdx.x * kVecThreads + threadIdx.x) * VEC; i < plane; i += (size_t)gridDim.x * kVecThreads * VEC) {
+
+// s = g / w_n in place, p = s, t = p / w_n, (s, s)
+template <typename R, int VEC>
+__global__ void __launch_bounds__(kVecThreads) cgls_first_model(const R* __restrict__ wm, R* __restrict__ g, R* __restrict__ p,
+                                                                R* __restrict__ t, size_t plane, int nz, Dot* ss, Dot* pp) {
+    using P = Pack<R, VEC>;
+    Squares<R> sum;
+    GRAV_FOR_LAYERS
+            P gv = *reinterpret_cast<const P*>(g + base + i), tv;
+#pragma unroll
+            for (int j = 0; j < VEC; ++j) {
+                const R s = gv.v[j] / wn;
+                gv.v[j] = s;
+                tv.v[j] = s / wn;
+                sum.add(s);
+            }
+            *reinterpret_cast<P*>(p + base + i) = gv;
+            *reinterpret_cast<P*>(t + base + i) = tv;
+        }
+    }
+    put_dot(ss, sum.get());
+    put_dot(pp, sum.get());
+}
+
+// x += alpha p (x = alpha p in the first step), s = g / w_n - lam x in place
+// of g, (s, s), (x, x); m = x / w_n if wanted
+template <typename R, int VEC>
+__global__ void __launch_bounds__(kVecThreads) cgls_step_model(Scalars k, bool first, const R* __restrict__ wm, const R* __restrict__ p, R* __restrict__ x,
+                                                               R* __restrict__ g, R* __restrict__ m, size_t plane, int nz,
+                                                               Dot* ss, Dot* xx) {
+    using P = Pack<R, VEC>;
+    const R alpha = (R)step_length(k), lam = (R)k.lam;
+    Squares<R> s2, x2;
+    GRAV_FOR_LAYERS
+            const P pv = *reinterpret_cast<const P*>(p + base + i);
+            P gv = *reinterpret_cast<const P*>(g + base + i), xv, mv;
+            if (first) {
+#pragma unroll
+                for (int j = 0; j < VEC; ++j) xv.v[j] = 0;
+            } else {
+                xv = *reinterpret_cast<const P*>(x + base + i);
+            }
+#pragma unroll
+            for (int j = 0; j < VEC; ++j) {
+                xv.v[j] += alpha * pv.v[j];
+                const R s = gv.v[j] / wn - lam * xv.v[j];
+                gv.v[j] = s;
+                mv.v[j] = xv.v[j] / wn;
+                s2.add(s);
+                x2.add(xv.v[j]);
+            }
+            *reinterpret_cast<P*>(x + base + i) = xv;
+            *reinterpret_cast<P*>(g + base + i) = gv;
+            if (m) *reinterpret_cast<P*>(m + base + i) = mv;
+        }
+    }
+    put_dot(ss, s2.get());
+    put_dot(xx, x2.get());
+}
+
+// p = s + beta p, t = p / w_n, (p, p)
+template <typename R, int VEC>
+__global__ void __launch_bounds__(kVecThreads) cgls_next_dir(const Dot* gamma, const Dot* gamma_new, const R* __restrict__ wm,
+                                                             const R* __restrict__ s, R* __restrict__ p, R* __restrict__ t,
+                                                             size_t plane, int nz, Dot* pp) {
+    using P = Pack<R, VEC>;
+    __shared__ double beta_sh;
+    if (threadIdx.x == 0) beta_sh = gamma->value == 0.0 ? 0.0 : gamma_new->value / gamma->value;
+    __syncthreads();
+    const R beta = (R)beta_sh;
+    Squares<R> p2;
+    GRAV_FOR_LAYERS
+            const P sv = *reinterpret_cast<const P*>(s + base + i);
+            P pv = *reinterpret_cast<const P*>(p + base + i), tv;
+#pragma unroll
+            for (int j = 0; j < VEC; ++j) {
+                pv.v[j] = sv.v[j] + beta * pv.v[j];
+                tv.v[j] = pv.v[j] / wn;
+                p2.add(pv.v[j]);
+            }
+            *reinterpret_cast<P*>(p + base + i) = pv;
+            *reinterpret_cast<P*>(t + base + i) = tv;
+        }
+    }
+    put_dot(pp, p2.get());
+}
+#undef GRAV_FOR_LAYERS
+
+// objectives[k] = (r, r) + lam (x, x) after k steps; dots: (r, r), (x, x), (s, s) per step
+__global__ void __launch_bounds__(kVecThreads) cgls_objectives(const Dot* dots, int n, double lam, double* __restrict__ obj) {
+    for (int k = threadIdx.x; k < n; k += kVecThreads) obj[k] = dots[3 * k].value + (k ? lam * dots[3 * k + 1].value : 0.0);
+}
+
+size_t pad256(size_t v) { return (v + 255) / 256 * 256; }
+
+// The caller's workspace: data vectors r, q, wr; model vectors p, t, g, x; then
+// the dot products: (p, p), (q, q) and, per step, (r, r), (x, x), (s, s).
+struct Work {
+    size_t nd, plane, data, model;
+    int nz, iters;
+    size_t dots() const { return 2 + 3 * ((size_t)iters + 1); }
+    size_t bytes() const { return 3 * data + 4 * model + dots() * sizeof(Dot); }
+};
+Work work_of(const grav_plan* p, int iters) {
+    Work w{};
+    const size_t real = p->fp64 ? 8 : 4;
+    w.plane = (size_t)p->ny * p->nx;
+    w.nd = w.plane * p->ncomp;
+    w.nz = p->nz;
+    w.iters = iters;
+    w.data = pad256(w.nd * real);
+    w.model = pad256(w.plane * p->nz * real);
+    return w;
+}
+
+template <typename R> struct Loop {
+    Work k;
+    R *r, *q, *wr, *p, *t, *g, *x;
+    Dot *pp, *qq, *step;
+    unsigned gd;      // blocks of the data-size kernels
+    dim3 gm;          // blocks of the model-size kernels
+    bool vec;
+    Loop(const grav_plan* plan, int iters, void* work) : k(work_of(plan, iters)) {
+        unsigned char* b = (unsigned char*)work;
+        auto take = [&](size_t n) {
+            R* v = (R*)b;
+            b += n;
+            return v;
+        };
+        r = take(k.data), q = take(k.data), wr = take(k.data);
+        p = take(k.model), t = take(k.model), g = take(k.model), x = take(k.model);
+        pp = (Dot*)b;
+        qq = pp + 1;
+        step = pp + 2;
+        gd = (unsigned)std::min<size_t>((k.nd + kVecThreads - 1) / kVecThreads, kMaxParts / 2);
+        constexpr int V = 16 / sizeof(R);
+        vec = k.plane % V == 0;
+        const unsigned gy = (unsigned)std::min(k.nz, kMaxParts);
+        const size_t per = (size_t)kVecThreads * (vec ? V : 1);
+        const unsigned gx = (unsigned)std::min<size_t>((k.plane + per - 1) / per, kMaxParts / gy);
+        gm = dim3(gx, gy);
+    }
+    Dot* rr(int it) const { return step + (size_t)3 * it; }
+    Dot* xx(int it) const { return rr(it) + 1; }
+    Dot* ss(int it) const { return rr(it) + 2; }
+};
+
+template <typename R>
+int run_start(grav_plan* plan, const R* d, const R* w, const R* wm, int iters, void* work, cudaStream_t s) {
+    const Loop<R> L(plan, iters, work);
+    constexpr int V = 16 / sizeof(R);
+    cudaError_t e = cudaMemsetAsync(L.pp, 0, L.k.dots() * sizeof(Dot), s);  // no block done yet
+    if (e != cudaSuccess) return cuda_fail(e, "grav_cgls_start");
+    cgls_first_data<R><<<L.gd, kVecThreads, 0, s>>>(d, w, L.r, L.wr, L.k.nd, L.rr(0));
+    const int rc = grav_adjoint(plan, L.wr, L.g, s);
+    if (rc != GRAV_OK) return rc;
+    if (L.vec) cgls_first_model<R, V><<<L.gm, kVecThreads, 0, s>>>(wm, L.g, L.p, L.t, L.k.plane, L.k.nz, L.ss(0), L.pp);
+    else cgls_first_model<R, 1><<<L.gm, kVecThreads, 0, s>>>(wm, L.g, L.p, L.t, L.k.plane, L.k.nz, L.ss(0), L.pp);
+    e = cudaGetLastError();
+    return e == cudaSuccess ? GRAV_OK : cuda_fail(e, "grav_cgls_start");
+}
+
+template <typename R>
+int run_steps(grav_plan* plan, const R* w, const R* wm, double lam, int iters, int keep, R* models, double* obj,
+              void* work, cudaStream_t s) {
+    const Loop<R> L(plan, iters, work);
+    constexpr int V = 16 / sizeof(R);
+    const size_t cells = L.k.plane * L.k.nz;
+    if (iters == 0 && !keep) {
+        const cudaError_t e = cudaMemsetAsync(models, 0, cells * sizeof(R), s);
+        if (e != cudaSuccess) return cuda_fail(e, "grav_cgls_steps");
+    }
+    for (int it = 0; it < iters; ++it) {
+        int rc = grav_forward(plan, L.t, L.q, s);
+        if (rc != GRAV_OK) return rc;
+        cgls_weigh<R><<<L.gd, kVecThreads, 0, s>>>(w, L.q, L.k.nd, L.qq);
+        const Scalars k{L.ss(it), L.pp, L.qq, lam};
+        cgls_step_data<R><<<L.gd, kVecThreads, 0, s>>>(k, w, L.q, L.r, L.wr, L.k.nd, L.rr(it + 1));
+        rc = grav_adjoint(plan, L.wr, L.g, s);
+        if (rc != GRAV_OK) return rc;
+        R* m = keep ? models + (size_t)it * cells : it + 1 == iters ? models : nullptr;
+        if (L.vec) cgls_step_model<R, V><<<L.gm, kVecThreads, 0, s>>>(k, it == 0, wm, L.p, L.x, L.g, m, L.k.plane, L.k.nz, L.ss(it + 1), L.xx(it + 1));
+        else cgls_step_model<R, 1><<<L.gm, kVecThreads, 0, s>>>(k, it == 0, wm, L.p, L.x, L.g, m, L.k.plane, L.k.nz, L.ss(it + 1), L.xx(it + 1));
+        if (it + 1 < iters) {
+            if (L.vec) cgls_next_dir<R, V><<<L.gm, kVecThreads, 0, s>>>(L.ss(it), L.ss(it + 1), wm, L.g, L.p, L.t, L.k.plane, L.k.nz, L.pp);
+            else cgls_next_dir<R, 1><<<L.gm, kVecThreads, 0, s>>>(L.ss(it), L.ss(it + 1), wm, L.g, L.p, L.t, L.k.plane, L.k.nz, L.pp);
+        }
+    }
+    cgls_objectives<<<1, kVecThreads, 0, s>>>(L.step, iters + 1, lam, obj);
+    const cudaError_t e = cudaGetLastError();
+    return e == cudaSuccess ? GRAV_OK : cuda_fail(e, "grav_cgls_steps");
+}
+
+int check_cgls(const grav_plan* plan, bool pointers, int iters, const void* work, const char* name) {
+    if (!plan || !pointers || !work || iters < 0) {
+        set_error("%s: null plan or buffer, or a negative number of steps", name);
+        return GRAV_EINVAL;
+    }
+    if (plan->kind != 0) {
+        set_error("%s: the plan was made by grav_plan_create3d", name);
+        return GRAV_EINVAL;
+    }
+    if (reinterpret_cast<uintptr_t>(work) & 255) {
+        set_error("%s: workspace must be 256-byte aligned", name);
+        return GRAV_EINVAL;
+    }
+    return GRAV_OK;
+}
+
+}  // namespace
+
+}  // namespace grav
+
+using namespace grav;
+
+extern "C" {
+
+size_t grav_cgls_work_bytes(const grav_plan* plan, int iters) {
+    return plan && plan->kind == 0 && iters >= 0 ? work_of(plan, iters).bytes() : 0;
+}
+
+int grav_cgls_start(grav_plan* plan, const void* d_dev, const void* w_dev, const void* wm_dev, int iters, void* work_dev,
+                    void* stream) {
+    const int rc = check_cgls(plan, d_dev && w_dev && wm_dev, iters, work_dev, "grav_cgls_start");
+    if (rc != GRAV_OK) return rc;
+    cudaStream_t s = (cudaStream_t)stream;
+    return plan->fp64 ? run_start<double>(plan, (const double*)d_dev, (const double*)w_dev, (const double*)wm_dev, iters, work_dev, s)
+                      : run_start<float>(plan, (const float*)d_dev, (const float*)w_dev, (const float*)wm_dev, iters, work_dev, s);
+}
+
+int grav_cgls_steps(grav_plan* plan, const void* w_dev, const void* wm_dev, double lam, int iters, int keep_models,
+                    void* models_dev, double* objectives_dev, void* work_dev, void* stream) {
+    const int rc = check_cgls(plan, w_dev && wm_dev && objectives_dev && (models_dev || (keep_models && iters == 0)), iters,
+                              work_dev, "grav_cgls_steps");
+    if (rc != GRAV_OK) return rc;
+    if (reinterpret_cast<uintptr_t>(models_dev) & 15) {
+        set_error("grav_cgls_steps: models must be 16-byte aligned");
+        return GRAV_EINVAL;
+    }
+    cudaStream_t s = (cudaStream_t)stream;
+    return plan->fp64 ? run_steps<double>(plan, (const double*)w_dev, (const double*)wm_dev, lam, iters, keep_models,
+                                          (double*)models_dev, objectives_dev, work_dev, s)
+                      : run_steps<float>(plan, (const float*)w_dev, (const float*)wm_dev, lam, iters, keep_models,
+                                         (float*)models_dev, objectives_dev, work_dev, s);
+}
+
+}  // extern "C"

@@ -30,6 +30,7 @@ from dataclasses import dataclass
 
 import torch
 
+from . import capi
 from .plan import Plan
 
 
@@ -108,6 +109,46 @@ def _dot(a: torch.Tensor, b: torch.Tensor) -> float:
     return float(torch.sum(a * b, dtype=torch.float64))
 
 
+def _on_device(plan, d: torch.Tensor, w, lam) -> bool:
+    """Whether the loop's operands are what grav_cgls_start / grav_cgls_steps
+    take: a plane plan itself (not a subclass or instance with products of its
+    own) and plain tensors of its type and device; anything else runs the loop
+    below operation by operation."""
+    return (type(plan) is Plan and not {"forward", "adjoint"} & vars(plan).keys()
+            and type(d) is torch.Tensor and type(w) is torch.Tensor
+            and isinstance(lam, (int, float)) and d.device == plan.device == w.device
+            and d.dtype == plan.dtype == w.dtype and tuple(d.shape) == (plan.ncomp, plan.ny, plan.nx)
+            and w.dim() <= 3 and all(a in (1, b) for a, b in zip(w.shape[::-1], d.shape[::-1]))
+            and not (d.requires_grad or w.requires_grad))
+
+
+def _cgls_on_device(plan: Plan, d, w, wm, lam: float, iters: int, keep_models: bool) -> CGLSResult:
+    """The loop below, enqueued whole by the library: one read of the
+    objectives at the end is the only wait."""
+    nx, ny, nz = plan.mesh[:3]
+    n = max(0, iters)
+    d = d.contiguous()
+    w = w.expand(d.shape).contiguous()
+    wm1 = wm.reshape(-1).contiguous()
+    work = torch.empty(capi.grav_cgls_work_bytes(plan.handle, n) + 256, dtype=torch.uint8, device=d.device)
+    base = (work.data_ptr() + 255) // 256 * 256
+    keep = keep_models and n > 0
+    models = torch.empty((n if keep else 1, nz, ny, nx), dtype=d.dtype, device=d.device)
+    obj = torch.empty(n + 1, dtype=torch.float64, device=d.device)
+    s = torch.cuda.current_stream(d.device)
+    e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    capi.grav_cgls_start(plan.handle, d.data_ptr(), w.data_ptr(), wm1.data_ptr(), n, base, s.cuda_stream)
+    e0.record(s)
+    capi.grav_cgls_steps(plan.handle, w.data_ptr(), wm1.data_ptr(), lam, n, keep, models.data_ptr(), obj.data_ptr(), base,
+                         s.cuda_stream)
+    e1.record(s)
+    m = models[-1].clone() if keep else models[0]
+    objectives = obj.tolist()
+    torch.cuda.synchronize()
+    return CGLSResult(m=m, models=list(models.unbind(0)) if keep else [], objectives=objectives,
+                      iterations=iters, lam=lam, ms_per_iteration=e0.elapsed_time(e1) / max(1, iters))
+
+
 def cgls(plan: Plan, d: torch.Tensor, w: torch.Tensor, lam: float, iters: int = 10, beta: float = 2.0,
          keep_models: bool = False) -> CGLSResult:
     """Damped CGLS with depth weights (see the module docstring).
@@ -118,6 +159,8 @@ def cgls(plan: Plan, d: torch.Tensor, w: torch.Tensor, lam: float, iters: int = 
     Returns the model m = W_m^-1 x and the objective after every iteration;
     ms_per_iteration is timed with CUDA events when d is on a GPU (else nan)."""
     wm = depth_weights(plan.mesh, beta, device=d.device, dtype=d.dtype)
+    if _on_device(plan, d, w, lam):
+        return _cgls_on_device(plan, d, w, wm, lam, iters, keep_models)
 
     def A(x):
         return w * plan.forward((x / wm).contiguous())
