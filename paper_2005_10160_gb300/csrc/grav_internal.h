@@ -227,9 +227,9 @@ cudaError_t launch_row_c2r_group(int log_p, const void* in0, const void* in1, in
 // more than 7 components) or err is null, and the caller takes another kernel.
 cudaError_t launch_forward_wf512(const ColumnArgs& a, const void* X, const float* spec, void* Y, const void* tw,
                                  int* err, cudaStream_t s, Batch b);
-// The adjoint counterpart (col_adj512_f32.cu), writing the untiled column
-// output; cudaErrorNotSupported when ny_pad > 512, more than 8 components,
-// err is null or a.z_tiled is set.
+// The adjoint counterpart (col_adj512_f32.cu), writing the summed column
+// output (a.z_summed); takes every plan with 512-point FP32 columns, and
+// returns cudaErrorInvalidValue for arguments that are not of one.
 cudaError_t launch_adjoint_wf512(const ColumnArgs& a, const void* Xr, const float* spec, void* Z, const void* tw,
                                  int* err, cudaStream_t s, Batch b);
 
@@ -242,7 +242,7 @@ cudaError_t launch_adjoint_groups(int log_n, const ColumnArgs& a, const void* Xr
                                   const void* tw, cudaStream_t s, Batch b);
 // Whether the FP32 adjoint column stage of 2^log_n-point columns adds the two
 // ky parities itself and writes Z[kx][n][y].
-constexpr bool adjoint_summed(int log_n) { return log_n >= 6 && log_n <= 8; }
+constexpr bool adjoint_summed(int log_n) { return log_n >= 6 && log_n <= 9; }
 
 // Adjoint inverse rows from the tiled column output (ColumnArgs::z_tiled):
 // in_r[n][y / 8][kx][8] (swizzled as described there) for r = 0, 1 (in1 = in0 + one half), summed, kx
