@@ -220,6 +220,16 @@ cudaError_t launch_row_r2c_group(int log_p, const float* in, size_t in_ostride, 
 cudaError_t launch_row_c2r_group(int log_p, const void* in0, const void* in1, int I, int O, int i_pad, float* out,
                                  size_t out_stride, int l_out, const void* tw, int log_t, cudaStream_t s, Batch b);
 
+// FP32 transforms of `rows` contiguous complex rows (the y passes of the
+// equal-dimension plans), row_groups.cu: forward, l_in <= P / 2 values
+// zero-padded to P = 2^log_p = 128 .. 2048; inverse, the first l_out <= P / 2
+// of P = 128 .. 2048 outputs kept.  Strides in complex elements;
+// cudaErrorNotSupported when the sizes or alignments do not fit.
+cudaError_t launch_rows_fwd_group(int log_p, const void* in, size_t in_stride, int l_in, void* out, size_t out_stride,
+                                  long rows, const void* tw, int log_t, cudaStream_t s);
+cudaError_t launch_rows_inv_group(int log_p, const void* in, size_t in_stride, void* out, size_t out_stride, int l_out,
+                                  long rows, const void* tw, int log_t, cudaStream_t s);
+
 // Forward column stage for 512-point FP32 columns (Py = 1024) with both ky
 // parities of a column in one CTA and two transforms per warp
 // (col_fwd512_f32.cu).  Same arguments and layouts as the column launchers

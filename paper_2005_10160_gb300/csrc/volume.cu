@@ -38,9 +38,11 @@
 // The adjoint runs the same passes from r[c][t][y][x], multiplies by the
 // conjugate spectra and sums over components in pass C (the transpose).
 // Generic block-FFT kernels serve every size; FP32 plans at the common sizes
-// take register-resident kernels instead: pass C for Pz = 256
-// (vol_z256_kernel), passes B and D for Py = 2048 (vol_yfwd2048_kernel,
-// vol_yinv2048_tiled_kernel) and, with Px = 2048, D writes the tiled layout
+// take register-resident kernels instead: pass C for Pz = 64 .. 256
+// (vol_zgroup_kernel), passes B and D for Py = 2048 (vol_yfwd2048_kernel,
+// vol_yinv2048_tiled_kernel) and for Py = 128 .. 1024 (and 2048 untiled;
+// launch_rows_fwd_group and launch_rows_inv_group of row_groups.cu) and, with
+// Px = 2048, D writes the tiled layout
 // V[c t][y / 8][kx][8] that pass E reads by bulk copies
 // (launch_row_c2r_tiled).
 #include <algorithm>
@@ -50,6 +52,7 @@
 #include "async_copy.cuh"
 #include "fft_block.cuh"
 #include "grav_internal.h"
+#include "group_fft.cuh"
 #include "warp_fft.cuh"
 
 namespace grav {
@@ -423,38 +426,50 @@ __global__ void __launch_bounds__(z_threads(TI, LOGZ, sizeof(R) == 8), 2)
     }
 }
 
-// Pass C for Pz = 256 in FP32, transforms in registers.  A warp owns two
-// columns of the tile; lane L works on column L / 16 with q = L % 16 and
-// holds 16 of its values.  256 = 16 x 16 (the four-step form):
-//   forward  x[q + 16 n2] -> 16-point DFT over n2 -> twiddle W_256^(q k2)
-//            -> transpose through the warp's shared area (q <-> k2)
-//            -> 16-point DFT over n1: lane q = k2 holds X[k2 + 16 k1] with
-//            k1 = bitrev4(j) in register j;
-//   inverse  from that layout: 16-point DFT over k1 -> twiddle W_256^(-a k2)
+// Pass C for Pz = 64, 128 and 256 in FP32 (17 <= nz <= 128), transforms in
+// registers by groups of L = Pz / 16 lanes, 16 values a lane (group_fft.cuh).
+// Lane q of a group works on one column of the tile:
+//   forward  x[q + L n2] -> 16-point DFT over n2 -> twiddle W^(q k2)
+//            -> transpose through the group's shared area (q <-> k2)
+//            -> L-point DFTs over n1: register i L + j of lane q holds
+//            X[k2 + 16 k1] with k2 = q + L i, k1 = bitrev(j);
+//   inverse  from that layout: L-point DFTs over k1 -> twiddle W^(-a k2)
 //            -> transpose -> 16-point DFT over k2: lane q = a holds
-//            x[a + 16 b], b = bitrev4(j).
-// Pz = 256 >= 2 nz - 1 gives nz <= 128, so the inputs x[q + 16 n2] with
-// n2 >= 8 are zero (the first stage of the forward DFT only twiddles) and
-// the stations kept are x[a + 16 b] with b < 8 (the even registers: the last
-// stage of the inverse DFT keeps its sums).  Tiles of nz rows x 8 columns
-// (a CTA of four warps) move between HBM and shared memory in rows of 64
-// bytes; the CTA grid runs the ky tiles of one kx next to each other, so each
-// kx's spectra are read from HBM once and served from L2 to both halves of
-// every mirror pair.
-constexpr int kZ2Warps = 4, kZ2Ti = 2 * kZ2Warps, kZ2Threads = 32 * kZ2Warps;
-constexpr int kZ2Str = kZ2Ti + 1;              // staging tile row stride (complex)
-constexpr int kZ2TrStr = 17;                   // transpose area row stride
-constexpr int kZ2TrWarp = 2 * 16 * kZ2TrStr;   // complex values of a warp's transpose area
-constexpr int kZ2MaxNz = 128;
-constexpr int kZ2Stage = kZ2MaxNz * kZ2Str;    // complex values of one staging tile
-// spectra of one component for the tile's columns, one row of Pz/2 + 1 = 129
-// values per column (both mirror halves of kz read the same row), two
-// components in flight
-constexpr int kZ2SpS = 145;                    // floats per staged spectra row (129 used)
-constexpr int kZ2Spec = kZ2Ti * kZ2SpS;        // floats of one component's staged spectra
-constexpr size_t kZ2Smem = (size_t)(256 + kZ2Warps * kZ2TrWarp + 2 * kZ2Stage) * sizeof(float2) +
-                           (size_t)2 * kZ2Spec * sizeof(float);
-static_assert(kZ2Threads == 16 * kZ2Ti, "sixteen threads stage each spectra row");
+//            x[a + L b], b = bitrev4(j).
+// Pz >= 2 nz - 1 gives nz <= Pz / 2, so the inputs x[q + L n2] with n2 >= 8
+// are zero (the first stage of the forward DFT only twiddles) and the
+// stations kept are x[a + L b] with b < 8 (the even registers: the last
+// stage of the inverse DFT keeps its sums).  Tiles of nz rows x 2048 / Pz
+// columns (a CTA of four warps) move between HBM and shared memory in rows of
+// 64 to 256 bytes; the CTA grid runs the ky tiles of one kx next to each
+// other, so each kx's spectra are read from HBM once and served from L2 to
+// both halves of every mirror pair.
+// Adjoint at 384 x 320 x 64 (Pz = 128, six components): 755 us, 1670 us with
+// the block transforms of vol_z_kernel (2.3 GB: 0.34 ms at the copy rate).
+constexpr int kZgWarps = 4, kZgThreads = 32 * kZgWarps;
+template <int PZ> struct ZGroup {
+    static constexpr int V = 16, L = PZ / V;           // values a lane, lanes of a column
+    static constexpr bool SYM = L == V;                // W^(r c) tables of both directions coincide
+    static constexpr int TABS = SYM ? PZ : 2 * PZ;     // table entries
+    static constexpr int GPW = 32 / L;                 // columns of a warp
+    static constexpr int TI = kZgWarps * GPW;          // columns of the tile
+    static constexpr int STR = TI + 1;                 // staging tile row stride (complex)
+    static constexpr int FROW = L + 1, IROW = V + 1;   // transpose row strides, forward and inverse
+    // complex values of a group's transpose area; the groups of a 16-lane
+    // phase start L apart modulo 16
+    static constexpr int AREA = L == 16 ? V * FROW : (V * FROW + 15) / 16 * 16 + L;
+    static constexpr int MAXNZ = PZ / 2;
+    static constexpr int STAGE = MAXNZ * STR;          // complex values of one staging tile
+    // spectra of one component for the tile's columns, one row of Pz / 2 + 1
+    // values per column (both mirror halves of kz read the same row), two
+    // components in flight; the row stride spreads the columns of a warp over
+    // the banks
+    static constexpr int SPS = L == 16 ? 145 : PZ / 2 + L;
+    static constexpr int SPEC = TI * SPS;
+    static constexpr size_t smem = (size_t)(TABS + kZgWarps * GPW * AREA + 2 * STAGE) * sizeof(float2) +
+                                   (size_t)2 * SPEC * sizeof(float);
+    static_assert(kZgThreads == L * TI, "L threads stage each spectra row");
+};
 
 // 16-point DFT in registers, radix-2 decimation in frequency: natural order
 // in, u[j] = X[bitrev4(j)] out.  HALF: u[8..15] are zero on entry.  LOW:
@@ -481,197 +496,219 @@ template <bool INV, bool HALF, bool LOW> __device__ __forceinline__ void dft16r(
     }
 }
 
-template <bool ADJ>
-__global__ void __launch_bounds__(kZ2Threads, 16 / kZ2Warps)
-    vol_z256_kernel(ZArgs a, const float2* __restrict__ in, float2* __restrict__ out, const float* __restrict__ spec3,
-                    const float2* __restrict__ tw) {
+template <int PZ, bool ADJ>
+__global__ void __launch_bounds__(kZgThreads, 16 / kZgWarps)
+    vol_zgroup_kernel(ZArgs a, const float2* __restrict__ in, float2* __restrict__ out, const float* __restrict__ spec3,
+                      const float2* __restrict__ tw) {
+    using S = ZGroup<PZ>;
+    constexpr int V = S::V, L = S::L, TI = S::TI, STR = S::STR;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    float2* tab = reinterpret_cast<float2*>(smem_raw);  // tab[r * 16 + c] = W_256^(r c)
+    float2* ftab = reinterpret_cast<float2*>(smem_raw);  // ftab[k2 L + q] = W^(q k2)
+    float2* itab = S::SYM ? ftab : ftab + PZ;            // itab[a V + k2] = W^(a k2)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int col = lane >> 4, q = lane & 15;
-    float2* tr = tab + 256 + warp * kZ2TrWarp + col * 16 * kZ2TrStr;  // this column's transpose area
-    float2* stage = tab + 256 + kZ2Warps * kZ2TrWarp;                 // two [t][kZ2Str] tiles
-    const int ky0 = blockIdx.x * kZ2Ti, kx = blockIdx.y;
+    const int col = lane / L, q = lane % L;
+    float2* tr = ftab + S::TABS + (warp * S::GPW + col) * S::AREA;  // this column's transpose area
+    float2* stage = ftab + S::TABS + kZgWarps * S::GPW * S::AREA;   // two [t][STR] tiles
+    const int ky0 = blockIdx.x * TI, kx = blockIdx.y;
     const int nz = a.nz, py = a.py;
-    const int ci = 2 * warp + col, ky = ky0 + ci;
+    const int ci = S::GPW * warp + col, ky = ky0 + ci;
     const bool fy = ky > py / 2;
 
-    for (int e = tid; e < 256; e += kZ2Threads) tab[e] = tw[((e >> 4) * (e & 15)) << a.tw_shift];
+    for (int e = tid; e < PZ; e += kZgThreads) {
+        ftab[e] = tw[((e / L) * (e % L)) << a.tw_shift];
+        if (!S::SYM) itab[e] = tw[((e / V) * (e % V)) << a.tw_shift];
+    }
 
-    // nz rows of the tile's 16 columns (zero beyond py) into a staging tile
-    // A thread moves column ti = tid % kZ2Ti of the tile, rows tr0, tr0 +
-    // kZ2Rs, ...: its shared and global addresses advance by fixed strides.
-    constexpr int kZ2Rs = kZ2Threads / kZ2Ti;  // rows per pass of the CTA
-    const int ti = tid % kZ2Ti, tr0 = tid / kZ2Ti;
+    // A thread moves column ti = tid % TI of the tile (zero beyond py), rows
+    // tr0, tr0 + RS, ...: its shared and global addresses advance by fixed
+    // strides.
+    constexpr int RS = kZgThreads / TI;  // rows per pass of the CTA
+    const int ti = tid % TI, tr0 = tid / TI;
     const bool ti_ok = ky0 + ti < py;
-    const size_t gstep = (size_t)kZ2Rs * py;
+    const size_t gstep = (size_t)RS * py;
     auto load_tile = [&](float2* st, const float2* src) {
-        float2* sp = st + tr0 * kZ2Str + ti;
+        float2* sp = st + tr0 * STR + ti;
         const float2* gp = src + (size_t)tr0 * py + ky0 + ti;
-        for (int n = tr0; n < nz; n += kZ2Rs, sp += kZ2Rs * kZ2Str, gp += gstep)
-            *sp = ti_ok ? *gp : make_float2(0.f, 0.f);
+        for (int n = tr0; n < nz; n += RS, sp += RS * STR, gp += gstep) *sp = ti_ok ? *gp : make_float2(0.f, 0.f);
     };
     // the same by per-thread asynchronous copies (one group per call)
     auto issue_tile = [&](float2* st, const float2* src) {
-        float2* sp = st + tr0 * kZ2Str + ti;
+        float2* sp = st + tr0 * STR + ti;
         const float2* gp = src + (size_t)tr0 * py + (ti_ok ? ky0 + ti : 0);
-        for (int n = tr0; n < nz; n += kZ2Rs, sp += kZ2Rs * kZ2Str, gp += gstep) async8_g2s(sp, gp, ti_ok);
+        for (int n = tr0; n < nz; n += RS, sp += RS * STR, gp += gstep) async8_g2s(sp, gp, ti_ok);
         async8_commit();
     };
     auto store_tile = [&](const float2* st, float2* dst) {
         if (!ti_ok) return;
-        const float2* sp = st + tr0 * kZ2Str + ti;
+        const float2* sp = st + tr0 * STR + ti;
         float2* gp = dst + (size_t)tr0 * py + ky0 + ti;
-        for (int t = tr0; t < nz; t += kZ2Rs, sp += kZ2Rs * kZ2Str, gp += gstep) *gp = *sp;
+        for (int t = tr0; t < nz; t += RS, sp += RS * STR, gp += gstep) *gp = *sp;
     };
     // forward transform of this lane's column from a staging tile
-    auto fwd_fft = [&](const float2* st, float2 (&u)[16]) {
+    auto fwd_fft = [&](const float2* st, float2 (&u)[V]) {
 #pragma unroll
-        for (int n2 = 0; n2 < 8; ++n2) {
-            const int n = q + 16 * n2;
-            u[n2] = n < nz ? st[n * kZ2Str + ci] : make_float2(0.f, 0.f);
+        for (int n2 = 0; n2 < V / 2; ++n2) {
+            const int n = q + L * n2;
+            u[n2] = n < nz ? st[n * STR + ci] : make_float2(0.f, 0.f);
         }
         dft16r<false, true, false>(u);
 #pragma unroll
-        for (int j = 0; j < 16; ++j) {
+        for (int j = 0; j < V; ++j) {
             const int k2 = bitrev4(j);
-            tr[k2 * kZ2TrStr + q] = cmul(u[j], tab[k2 * 16 + q]);
+            tr[k2 * S::FROW + q] = cmul(u[j], ftab[k2 * L + q]);
         }
         __syncwarp();
 #pragma unroll
-        for (int n1 = 0; n1 < 16; ++n1) u[n1] = tr[q * kZ2TrStr + n1];
+        for (int i = 0; i < V / L; ++i) {
+#pragma unroll
+            for (int n1 = 0; n1 < L; ++n1) u[i * L + n1] = tr[(q + L * i) * S::FROW + n1];
+        }
         __syncwarp();
-        dft16r<false, false, false>(u);
+#pragma unroll
+        for (int i = 0; i < V / L; ++i) dft_regs<L, false>(u + i * L);
     };
-    // inverse transform in place; the stations t = q + 16 bitrev4(j) < 128
+    // the forward keeps the inverse transform's twiddles in registers over the
+    // components (1024 x 1024 x 100: 12.27 -> 11.82 ms for the whole forward)
+    float2 wi[V];
+    if constexpr (!ADJ) {
+        __syncthreads();  // the tables are in place
+#pragma unroll
+        for (int e = 0; e < V; ++e) wi[e] = cconj(itab[bitrev_m<L>(e % L) * V + q + L * (e / L)]);
+    }
+    // inverse transform in place; the stations t = q + L bitrev4(j) < Pz / 2
     // are in the even registers j on exit
-    auto inv_fft = [&](float2 (&g)[16]) {
-        float2 h[16];
+    auto inv_fft = [&](float2 (&g)[V]) {
+        float2 h[V];
 #pragma unroll
-        for (int k1 = 0; k1 < 16; ++k1) h[k1] = g[bitrev4(k1)];
-        dft16r<true, false, false>(h);
+        for (int i = 0; i < V / L; ++i) {
 #pragma unroll
-        for (int j = 0; j < 16; ++j) {
-            const int aa = bitrev4(j);
-            tr[aa * kZ2TrStr + q] = cmul(h[j], cconj(tab[aa * 16 + q]));
+            for (int k1 = 0; k1 < L; ++k1) h[i * L + k1] = g[i * L + bitrev_m<L>(k1)];
+            dft_regs<L, true>(h + i * L);
+#pragma unroll
+            for (int j = 0; j < L; ++j) {
+                const int aa = bitrev_m<L>(j), k2 = q + L * i;
+                tr[aa * S::IROW + k2] = cmul(h[i * L + j], ADJ ? cconj(itab[aa * V + k2]) : wi[i * L + j]);
+            }
         }
         __syncwarp();
 #pragma unroll
-        for (int k2 = 0; k2 < 16; ++k2) g[k2] = tr[q * kZ2TrStr + k2];
+        for (int k2 = 0; k2 < V; ++k2) g[k2] = tr[q * S::IROW + k2];
         __syncwarp();
         dft16r<true, false, true>(g);
     };
-    auto put_stations = [&](float2* st, const float2 (&g)[16]) {
+    auto put_stations = [&](float2* st, const float2 (&g)[V]) {
 #pragma unroll
-        for (int j = 0; j < 16; j += 2) {
-            const int t = q + 16 * bitrev4(j);
-            if (t < nz) st[t * kZ2Str + ci] = g[j];
+        for (int j = 0; j < V; j += 2) {
+            const int t = q + L * bitrev4(j);
+            if (t < nz) st[t * STR + ci] = g[j];
         }
     };
-    // spectrum of slot c at (ky, kz = q + 16 bitrev4(j)) as the real v with
-    // S = v or S = i v
     // Spectra come into shared memory by per-thread asynchronous copies one
-    // component ahead: thread tid stages row sr = tid / 16 (column ky0 + sr)
-    // at jz = tid % 16 + 16 m; a row beyond py is zero-filled.
-    float* specb = reinterpret_cast<float*>(stage + 2 * kZ2Stage);  // two [kZ2Ti][kZ2SpS]
-    const int sr = tid >> 4, sz = tid & 15;
+    // component ahead: thread tid stages row sr = tid / L (column ky0 + sr)
+    // at jz = tid % L + L m; a row beyond py is zero-filled.
+    float* specb = reinterpret_cast<float*>(stage + 2 * S::STAGE);  // two [TI][SPS]
+    const int sr = tid / L, sz = tid % L;
     const int sky = ky0 + sr;
     const bool s_ok = sky < py;
     const float* spec_row = spec3 + ((size_t)kx * a.jyc + (!s_ok ? 0 : (sky > py / 2 ? py - sky : sky))) * a.jzc;
     const size_t spec_slot = (size_t)a.kx_count * a.jyc * a.jzc;
     auto issue_spec = [&](int c, float* sb) {
         const float* src = spec_row + c * spec_slot + sz;
-        uint32_t dst = smem_u32(sb + sr * kZ2SpS + sz);
+        uint32_t dst = smem_u32(sb + sr * S::SPS + sz);
         const uint32_t nb = s_ok ? 4u : 0u;
 #pragma unroll
         for (int m = 0; m < 9; ++m) {
-            if (m < 8 || sz == 0)  // jz = sz + 16 m <= 128
-                asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst + 64u * m), "l"(src + 16 * m),
+            if (m < 8 || sz == 0)  // jz = sz + L m <= Pz / 2
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst + 4u * L * m), "l"(src + L * m),
                              "r"(nb)
                              : "memory");
         }
         async8_commit();
     };
-    // spectrum of slot c at (ky, kz = q + 16 bitrev4(j)) from staged row ci
-    auto load_spec = [&](int c, const float* sb, float (&v)[16]) {
-        const float* row = sb + ci * kZ2SpS;
-        // the sign of S(ky, kz) against the stored value: flipped by the
-        // y parity for ky > Py/2 and by the w parity for kz > Pz/2
+    // f(e, v) for every register e with S = v (or i v) the spectrum of slot c at
+    // its (ky, kz), from staged row ci.  The stored value is negated by the y
+    // parity for ky > Py/2 and by the w parity for kz > Pz/2; registers with
+    // k1 < L / 2 have kz < Pz/2, the others kz > Pz/2 or the bin Pz/2, whose
+    // spectrum is 0 for components odd in w.  Both signs are the same for all
+    // lanes but in the tile that holds ky = Py/2, so they become compile-time
+    // variants.
+    auto with_spec = [&](int c, const float* sb, auto f) {
+        const float* row = sb + ci * S::SPS;
         const bool s_lo = fy && ((a.oddv_mask >> c) & 1u);
         const bool s_hi = s_lo != (((a.oddw_mask >> c) & 1u) != 0);
+        auto each = [&](auto lo, auto hi) {
 #pragma unroll
-        for (int j = 0; j < 16; ++j) {
-            const int kz = q + 16 * bitrev4(j);
-            const bool fz = kz > 128;
-            const float val = row[fz ? 256 - kz : kz];
-            v[j] = (fz ? s_hi : s_lo) ? -val : val;
-        }
+            for (int e = 0; e < V; ++e) {
+                const int k1 = bitrev_m<L>(e % L), kz = q + L * (e / L) + V * k1;
+                const bool up = 2 * k1 >= L;
+                const float val = row[up ? PZ - kz : kz];
+                f(e, (up ? hi() : lo()) ? -val : val);
+            }
+        };
+        const unsigned sides = __ballot_sync(0xffffffffu, fy);
+        if (sides != 0 && sides != 0xffffffffu) each([&] { return s_lo; }, [&] { return s_hi; });
+        else if (s_lo && s_hi) each([] { return true; }, [] { return true; });
+        else if (s_lo) each([] { return true; }, [] { return false; });
+        else if (s_hi) each([] { return false; }, [] { return true; });
+        else each([] { return false; }, [] { return false; });
     };
 
     if constexpr (!ADJ) {
-        float2* st_in = stage + kZ2Stage;
+        float2* st_in = stage + S::STAGE;
         issue_spec(0, specb);
         load_tile(st_in, in + (size_t)kx * nz * py);
         async8_wait_all();
-        __syncthreads();  // the tile, component 0's spectra and the twiddle table are in place
-        float2 X[16];
+        __syncthreads();  // the tile, component 0's spectra and the twiddle tables are in place
+        float2 X[V];
         fwd_fft(st_in, X);
         for (int c = 0; c < a.ncomp; ++c) {
             // the other spectra buffer was last read by component c - 1,
             // before the previous barrier
-            if (c + 1 < a.ncomp) issue_spec(c + 1, specb + ((c + 1) & 1) * kZ2Spec);
-            float v[16];
-            load_spec(c, specb + (c & 1) * kZ2Spec, v);
-            float2 g[16];
-            if ((a.imag3_mask >> c) & 1u) {  // S = i v
-#pragma unroll
-                for (int j = 0; j < 16; ++j) g[j] = make_float2(-v[j] * X[j].y, v[j] * X[j].x);
-            } else {
-#pragma unroll
-                for (int j = 0; j < 16; ++j) g[j] = make_float2(v[j] * X[j].x, v[j] * X[j].y);
-            }
+            if (c + 1 < a.ncomp) issue_spec(c + 1, specb + ((c + 1) & 1) * S::SPEC);
+            float2 g[V];
+            const float* sb = specb + (c & 1) * S::SPEC;
+            if ((a.imag3_mask >> c) & 1u)  // S = i v
+                with_spec(c, sb, [&](int e, float v) { g[e] = make_float2(-v * X[e].y, v * X[e].x); });
+            else
+                with_spec(c, sb, [&](int e, float v) { g[e] = make_float2(v * X[e].x, v * X[e].y); });
             inv_fft(g);
             // staging tile c % 2: its last reader (the store of component
             // c - 2, or the input read for c = 1) finished before the
             // previous barrier
-            float2* st = stage + (c & 1) * kZ2Stage;
+            float2* st = stage + (c & 1) * S::STAGE;
             put_stations(st, g);
             async8_wait_all();  // component c + 1's spectra, visible after the barrier
             __syncthreads();
             store_tile(st, out + ((size_t)kx * a.ncomp + c) * nz * py);
         }
     } else {
-        float2 acc[16];
+        float2 acc[V];
 #pragma unroll
-        for (int j = 0; j < 16; ++j) acc[j] = make_float2(0.f, 0.f);
+        for (int j = 0; j < V; ++j) acc[j] = make_float2(0.f, 0.f);
         // component c's tile is copied into staging tile c % 2 while
         // component c - 1 is transformed
         issue_tile(stage, in + (size_t)kx * a.ncomp * nz * py);
         issue_spec(0, specb);
         for (int c = 0; c < a.ncomp; ++c) {
-            float2* st = stage + (c & 1) * kZ2Stage;
+            float2* st = stage + (c & 1) * S::STAGE;
             async8_wait_all();
             // tile c and its spectra have landed everywhere, and every read of
             // tile c - 1 and its spectra (the other buffers) is done
             __syncthreads();
             if (c + 1 < a.ncomp) {
-                issue_tile(stage + ((c + 1) & 1) * kZ2Stage, in + ((size_t)kx * a.ncomp + c + 1) * nz * py);
-                issue_spec(c + 1, specb + ((c + 1) & 1) * kZ2Spec);
+                issue_tile(stage + ((c + 1) & 1) * S::STAGE, in + ((size_t)kx * a.ncomp + c + 1) * nz * py);
+                issue_spec(c + 1, specb + ((c + 1) & 1) * S::SPEC);
             }
-            float2 f[16];
+            float2 f[V];
             fwd_fft(st, f);
-            float v[16];
-            load_spec(c, specb + (c & 1) * kZ2Spec, v);
-            if ((a.imag3_mask >> c) & 1u) {  // conj(S) f with S = i v
-#pragma unroll
-                for (int j = 0; j < 16; ++j) acc[j] = make_float2(acc[j].x + v[j] * f[j].y, acc[j].y - v[j] * f[j].x);
-            } else {  // S = v
-#pragma unroll
-                for (int j = 0; j < 16; ++j) acc[j] = make_float2(acc[j].x + v[j] * f[j].x, acc[j].y + v[j] * f[j].y);
-            }
+            const float* sb = specb + (c & 1) * S::SPEC;
+            if ((a.imag3_mask >> c) & 1u)  // conj(S) f with S = i v
+                with_spec(c, sb, [&](int e, float v) { acc[e] = make_float2(acc[e].x + v * f[e].y, acc[e].y - v * f[e].x); });
+            else
+                with_spec(c, sb, [&](int e, float v) { acc[e] = make_float2(acc[e].x + v * f[e].x, acc[e].y + v * f[e].y); });
         }
         inv_fft(acc);
-        float2* st = stage + (a.ncomp & 1) * kZ2Stage;  // not the tile the last component read
+        float2* st = stage + (a.ncomp & 1) * S::STAGE;  // not the tile the last component read
         put_stations(st, acc);
         __syncthreads();
         store_tile(st, out + (size_t)kx * nz * py);
@@ -845,17 +882,34 @@ cudaError_t launch_vol_yfwd(int logn, const void* in, size_t in_stride, int l_in
             return cudaGetLastError();
         }
     }
+    if constexpr (std::is_same<C, float2>::value) {
+        const cudaError_t e = launch_rows_fwd_group(logn, in, in_stride, l_in, out, out_stride, rows, tw, log_t, s);
+        if (e != cudaErrorNotSupported) return e;
+    }
     return launch_vol_rows<C, false>(logn, in, in_stride, l_in, out, out_stride, (int)out_stride, rows, tw, log_t, s);
+}
+
+// Pass D (untiled): inverse column FFTs of `rows` rows of Py values, the
+// first l_out <= Py / 2 kept.
+template <typename C>
+cudaError_t launch_vol_yinv(int logn, const void* in, size_t in_stride, void* out, size_t out_stride, int l_out,
+                            long rows, const void* tw, int log_t, cudaStream_t s) {
+    if constexpr (std::is_same<C, float2>::value) {
+        const cudaError_t e = launch_rows_inv_group(logn, in, in_stride, out, out_stride, l_out, rows, tw, log_t, s);
+        if (e != cudaErrorNotSupported) return e;
+    }
+    return launch_vol_rows<C, true>(logn, in, in_stride, 1 << logn, out, out_stride, l_out, rows, tw, log_t, s);
 }
 
 template <typename R, int LOGZ, bool ADJ>
 cudaError_t z_launch(const ZArgs& a, const void* in, void* out, const R* spec3, const void* tw, cudaStream_t s) {
     using C = typename cplx<R>::type;
-    if constexpr (std::is_same<R, float>::value && LOGZ == 8) {
-        constexpr auto k = vol_z256_kernel<ADJ>;
+    if constexpr (std::is_same<R, float>::value && LOGZ >= 6 && LOGZ <= 8) {
+        using S = ZGroup<(1 << LOGZ)>;
+        constexpr auto k = vol_zgroup_kernel<(1 << LOGZ), ADJ>;
         cudaError_t e = ensure_smem_limit<k>();
         if (e != cudaSuccess) return e;
-        k<<<dim3((a.py + kZ2Ti - 1) / kZ2Ti, a.kx_count), kZ2Threads, kZ2Smem, s>>>(a, (const float2*)in, (float2*)out,
+        k<<<dim3((a.py + S::TI - 1) / S::TI, a.kx_count), kZgThreads, S::smem, s>>>(a, (const float2*)in, (float2*)out,
                                                                                    spec3, (const float2*)tw);
         return cudaGetLastError();
     } else {
@@ -1081,8 +1135,7 @@ int run_forward3d(grav_plan* p, const void* rho, void* out, cudaStream_t s) {
         }
     }
     // D: inverse y
-    e = launch_vol_rows<C, true>(p->log_py, A, p->py, p->py, B, p->ny_pad, p->ny, (long)(kx * nc * nz), p->tw,
-                                 p->log_t, s);
+    e = launch_vol_yinv<C>(p->log_py, A, p->py, B, p->ny_pad, p->ny, (long)(kx * nc * nz), p->tw, p->log_t, s);
     if (e != cudaSuccess) return cuda_fail(e, "equal-dimension forward: inverse column transforms");
     // E: inverse x
     e = launch_row_c2r<R>(p->log_px, B, nullptr, p->ny, (int)(nc * nz), p->ny_pad, (R*)out, (size_t)p->nx, p->nx,
@@ -1115,7 +1168,7 @@ int run_adjoint3d(grav_plan* p, const void* r, void* grad, cudaStream_t s) {
             return GRAV_OK;
         }
     }
-    e = launch_vol_rows<C, true>(p->log_py, A, p->py, p->py, B, p->ny_pad, p->ny, (long)(kx * nz), p->tw, p->log_t, s);
+    e = launch_vol_yinv<C>(p->log_py, A, p->py, B, p->ny_pad, p->ny, (long)(kx * nz), p->tw, p->log_t, s);
     if (e != cudaSuccess) return cuda_fail(e, "equal-dimension adjoint: inverse column transforms");
     e = launch_row_c2r<R>(p->log_px, B, nullptr, p->ny, p->nz, p->ny_pad, (R*)grad, (size_t)p->nx, p->nx, p->tw,
                           p->log_t, s);

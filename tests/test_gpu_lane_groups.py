@@ -9,7 +9,7 @@ import torch
 
 from paper_2005_10160_gb300 import capi
 from paper_2005_10160_gb300.batch import BatchRunner
-from paper_2005_10160_gb300.plan import Plan
+from paper_2005_10160_gb300.plan import Plan, Plan3D
 
 pytestmark = pytest.mark.gpu
 
@@ -58,3 +58,32 @@ def test_lane_group_kernels_match_the_fp64_path(gravlib, i, size):
         for k in range(3):
             assert torch.equal(db[k], plan.forward(rho[k]))
             assert torch.equal(gb[k], plan.adjoint(r[k]))
+
+
+MESHES3D = [
+    # Pz = 64 and 128 with the least and most layers, Py = 128 .. 1024 and 2048 (untiled inverse)
+    (20, 33, 17), (33, 64, 32), (40, 100, 33), (17, 257, 64), (65, 300, 40), (24, 40, 20), (30, 700, 18), (130, 129, 63),
+]
+
+
+@pytest.mark.parametrize("i,size", list(enumerate(MESHES3D)))
+def test_equal_dim_lane_groups_match_the_fp64_path(gravlib, i, size):
+    nx, ny, nz = size
+    mesh = (nx, ny, nz, 20.0, 25.0, 15.0)
+    comps = MASKS[i % len(MASKS)]
+    lst = capi.comp_list(comps)
+    first = torch.tensor([c in (0, 7, 8) for c in lst])
+    gen = torch.Generator(device="cuda").manual_seed(100 + i)
+    rho = torch.empty((nz, ny, nx), device="cuda").uniform_(-500, 500, generator=gen)
+    scale = torch.where(first, 1.0, 20.0).to("cuda")[:, None, None, None]
+    r = torch.empty((len(lst), nz, ny, nx), device="cuda").normal_(generator=gen) * scale
+    with Plan3D(mesh, comps) as plan, Plan3D(mesh, comps, fp64=True) as plan64:
+        d, g = plan.forward(rho), plan.adjoint(r)
+        d64, g64 = plan64.forward(rho.double()), plan64.adjoint(r.double())
+    diff, norm = worst(d, d64)
+    for kind in (True, False):
+        sel = (first == kind).to("cuda")
+        if sel.any():
+            floor = 1e-3 * norm[sel].max()
+            assert bool((diff[sel] <= TOL32 * torch.maximum(norm[sel], floor)).all()), (diff, norm)
+    assert float((g.double() - g64).norm()) <= TOL32 * float(g64.norm())
