@@ -15,6 +15,7 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <algorithm>
 #include <new>
 
 #include "grav_internal.h"
@@ -145,9 +146,9 @@ void free_plan(grav_plan* p) {
     delete p;
 }
 
-int build_twiddles(int log_t, int fp64, void** dev, size_t* bytes) {
+int build_twiddles(int log_t, int kind, void** dev, size_t* bytes) {
     const long T = 1L << log_t;
-    const size_t elem = fp64 ? 16 : 8;
+    const size_t elem = kind == kTwFloat ? 8 : 16;
     *bytes = (size_t)T * elem;
     unsigned char* host = (unsigned char*)malloc(*bytes);
     if (!host) {
@@ -157,9 +158,13 @@ int build_twiddles(int log_t, int fp64, void** dev, size_t* bytes) {
     for (long e = 0; e < T; ++e) {
         double re, im;
         unit_root(e, T, &re, &im);
-        if (fp64) {
+        if (kind == kTwDouble) {
             double* d = (double*)host + 2 * e;
             d[0] = re; d[1] = im;
+        } else if (kind == kTwPairs) {
+            float* f = (float*)host + 4 * e;
+            f[0] = (float)re; f[1] = (float)(re - (double)f[0]);
+            f[2] = (float)im; f[3] = (float)(im - (double)f[2]);
         } else {
             float* f = (float*)host + 2 * e;
             f[0] = (float)re; f[1] = (float)im;
@@ -176,63 +181,61 @@ int build_twiddles(int log_t, int fp64, void** dev, size_t* bytes) {
 
 namespace {
 
-template <typename R>
 int make_spectra(grav_plan* p) {
-    // FP64 staging: the embedded kernels of a chunk of layers and their row
-    // transforms, bounded to about 2 GB.
-    // rows b < py / 2 of each embedded kernel (the other half mirrors them)
-    const int hy = p->py / 2;
-    const size_t per_layer = (size_t)p->ncomp * hy * p->px * sizeof(double) +
-                             (size_t)p->kx_count * p->ncomp * hy * 2 * sizeof(double);
-    const size_t budget = (size_t)2 << 30;
-    int nzc = (int)(budget / per_layer);
+    // Staging: the quadrants of the embedded kernels of a chunk of layers and
+    // their row transforms, 8 bytes a value (FP64, or FP32 pairs), bounded to
+    // about 512 MB.
+    const int ny2 = (p->ny + 1) / 2 * 2;
+    const size_t e_layer = (size_t)p->ncomp * p->ny * p->nx * 8, t_layer = (size_t)p->kx_count * p->ncomp * ny2 * 8;
+    const size_t budget = (size_t)512 << 20;
+    int nzc = (int)std::min<size_t>(budget / (e_layer + t_layer), (size_t)p->nz);
     if (nzc < 1) nzc = 1;
-    if (nzc > p->nz) nzc = p->nz;
     if (nzc * p->ncomp > 65535) nzc = 65535 / p->ncomp;
+    const int chunks = (p->nz + nzc - 1) / nzc;  // of equal length
+    nzc = (p->nz + chunks - 1) / chunks;
 
-    void* tw64 = nullptr;
-    size_t tw64_bytes = 0;
+    void* tws = nullptr;
+    size_t tw_bytes = 0;
     int rc = GRAV_OK;
     if (p->fp64) {
-        tw64 = p->tw;
+        tws = p->tw;
     } else {
-        rc = build_twiddles(p->log_t, 1, &tw64, &tw64_bytes);
+        rc = build_twiddles(p->log_t, kTwPairs, &tws, &tw_bytes);
         if (rc) return rc;
     }
-    double* E = nullptr;
-    void* Ehat = nullptr;
-    const size_t e_bytes = (size_t)nzc * p->ncomp * hy * p->px * sizeof(double);
-    const size_t eh_bytes = (size_t)p->kx_count * nzc * p->ncomp * hy * 2 * sizeof(double);
-    if ((rc = dev_alloc(&E, e_bytes, "kernel staging")) == GRAV_OK &&
-        (rc = dev_alloc(&Ehat, eh_bytes, "kernel row-transform staging")) == GRAV_OK) {
+    void *E = nullptr, *T = nullptr;
+    if ((rc = dev_alloc(&E, nzc * e_layer, "kernel staging")) == GRAV_OK &&
+        (rc = dev_alloc(&T, nzc * t_layer, "kernel row-transform staging")) == GRAV_OK) {
         cudaStream_t s;
         cudaError_t ce = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
         if (ce != cudaSuccess) {
             rc = cuda_fail(ce, "cudaStreamCreate");
         } else {
-            Geometry g{p->nx, p->ny, p->nz, p->dx, p->dy, p->dz, p->h};
-            const double scale = 1.0 / ((double)p->px * (double)p->py);
+            const Geometry g{p->nx, p->ny, p->nz, p->dx, p->dy, p->dz, p->h};
+            SpecBuild b{p->nx, p->ny, p->nz, ny2, p->ncomp, p->kx_count, p->jp, p->log_px, p->log_py, 0, p->oddv_mask};
+            GenOut o = gen_out(p->fp64 ? GenOut::kQuadrant : GenOut::kQuadrantPairs);
+            double factor[kMaxPlanComp];
+            // FP32 pairs: kernels in units of upsilon (times the largest cell
+            // edge for first derivatives), which are of order 1 at most
+            const double edge = std::max(p->dx, std::max(p->dy, p->dz));
+            for (int slot = 0; slot < p->ncomp; ++slot) {
+                const int c = p->comp_id[slot];
+                if (odd_u(c)) b.oddu_mask |= 1u << slot;
+                factor[slot] = 1.0 / ((double)p->px * (double)p->py);
+                if (!p->fp64) {
+                    const double unit = first_derivative(c) ? edge : 1.0;
+                    o.factor[c] = 1.0 / unit;
+                    factor[slot] *= kUpsilon * unit;
+                }
+            }
             for (int n0 = 0; n0 < p->nz && rc == GRAV_OK; n0 += nzc) {
                 const int n1 = n0 + nzc < p->nz ? n0 + nzc : p->nz;
-                const int cnt = n1 - n0;
-                const int O = cnt * p->ncomp;
-                if ((ce = cudaMemsetAsync(E, 0, (size_t)O * hy * p->px * sizeof(double), s)) != cudaSuccess) {
-                    rc = cuda_fail(ce, "cudaMemsetAsync(kernel staging)");
-                    break;
-                }
-                if ((ce = launch_kernel_gen(g, p->comps, n0, n1, 2, p->px, p->py, E, s)) != cudaSuccess) {
+                if ((ce = launch_kernel_gen(g, o, p->comps, n0, n1, E, s)) != cudaSuccess) {
                     rc = cuda_fail(ce, "kernel generation launch");
                     break;
                 }
-                // rows o = slot * cnt + (n - n0) of length px, py / 2 of them per o
-                if ((ce = launch_row_r2c<double>(p->log_px, E, (size_t)hy * p->px, (size_t)p->px, p->px, hy, O,
-                                                 Ehat, hy, tw64, p->log_t, s)) != cudaSuccess) {
-                    rc = cuda_fail(ce, "kernel row transform launch");
-                    break;
-                }
-                if ((ce = launch_spec_extract<R>(p->log_py - 1, Ehat, p->kx_count, cnt, p->ncomp, n0, p->nz, p->jp,
-                                                 p->imag_mask, p->oddv_mask, scale, (R*)p->spec, tw64, p->log_t,
-                                                 s)) != cudaSuccess) {
+                if ((ce = launch_spec_build_chunk(b, p->fp64, E, n1 - n0, n0, T, factor, p->spec, tws, p->log_t, s)) !=
+                    cudaSuccess) {
                     rc = cuda_fail(ce, "kernel spectra launch");
                     break;
                 }
@@ -243,8 +246,8 @@ int make_spectra(grav_plan* p) {
         }
     }
     cudaFree(E);
-    cudaFree(Ehat);
-    if (!p->fp64) cudaFree(tw64);
+    cudaFree(T);
+    if (!p->fp64) cudaFree(tws);
     return rc;
 }
 
@@ -503,7 +506,7 @@ grav_plan* grav_plan_create(int nx, int ny, int nz, double dx, double dy, double
         cudaError_t me = cudaMemset(p->err_flag, 0, 256);
         if (me != cudaSuccess) rc = cuda_fail(me, "cudaMemset(error flag)");
     }
-    if (!rc) rc = p->fp64 ? make_spectra<double>(p) : make_spectra<float>(p);
+    if (!rc) rc = make_spectra(p);
     if (rc) {
         free_plan(p);
         return nullptr;
@@ -585,7 +588,7 @@ int grav_kernel_values(int nx, int ny, int nz, double dx, double dy, double dz, 
         return GRAV_EINVAL;
     }
     Geometry g{nx, ny, nz, dx, dy, dz, h};
-    cudaError_t e = launch_kernel_gen(g, components & kCompBits, 0, nz, 1, 0, 0, K_dev, (cudaStream_t)stream);
+    cudaError_t e = launch_kernel_gen(g, gen_out(GenOut::kOffsets), components & kCompBits, 0, nz, K_dev, (cudaStream_t)stream);
     if (e != cudaSuccess) return cuda_fail(e, "kernel generation launch");
     return GRAV_OK;
 }

@@ -25,6 +25,9 @@ constexpr unsigned kOddVMask = 0x124u;  // gxy, gyz, gy
 __host__ __device__ constexpr bool odd_u(int c) { return (kOddUMask >> c) & 1u; }
 __host__ __device__ constexpr bool odd_v(int c) { return (kOddVMask >> c) & 1u; }
 
+// gz, gx, gy are first derivatives of the potential, the rest second ones.
+__host__ __device__ constexpr bool first_derivative(int c) { return c == 0 || c == 7 || c == 8; }
+
 // Geometry shared by the kernel-generation launches.
 struct Geometry {
     int nx, ny, nz;
@@ -177,21 +180,33 @@ size_t round_up(size_t v, size_t m);
 // component mask are valid for a plan.
 int check_geometry(int nx, int ny, int nz, double dx, double dy, double dz, double h, unsigned components);
 int dev_alloc_raw(void** p, size_t bytes, const char* what);
-// Twiddle table W_T[e] = exp(-2 pi i e / T), T = 2^log_t, in FP64 (fp64 = 1)
-// or FP32, on the device.
-int build_twiddles(int log_t, int fp64, void** dev, size_t* bytes);
+// Twiddle table W_T[e] = exp(-2 pi i e / T), T = 2^log_t, on the device, in
+// FP32, FP64 or unevaluated pairs of FP32 (hi, lo per part).
+enum { kTwFloat = 0, kTwDouble = 1, kTwPairs = 2 };
+int build_twiddles(int log_t, int kind, void** dev, size_t* bytes);
 // Frees every device buffer and event of the plan, and the plan.
 void free_plan(grav_plan* p);
 
 // ---- kernel generation (kernel_gen.cu) ----
-// mode 0: embed into a circulant array E[(c * nzc + n) * py + b][a] of size
-//         py x px per (component, layer); E must be zeroed beforehand.
-// mode 2: the same, rows b < py / 2 only, E[(c * nzc + n) * (py / 2) + b][a]
-//         (the embedded kernel is even or odd in y, so row py - b is row b
-//         times the component's sign, and row py / 2 is zero).
-// mode 1: dense offset grid K[c][n][2ny-1][2nx-1].
-cudaError_t launch_kernel_gen(const Geometry& g, unsigned comps, int n0, int n1, int mode,
-                              int px, int py, double* out, cudaStream_t s);
+struct GenOut {
+    enum Mode {
+        kOffsets,        // dense offset grid K[c][n][2ny-1][2nx-1], all layers
+        kHalfRows,       // embedded circulant rows b < py / 2, E[(c * nzc + n) * (py / 2) + b][a], a < px;
+                         // E must be zeroed beforehand (the embedded kernel is even or odd in y, so row
+                         // py - b is row b times the component's sign, and row py / 2 is zero)
+        kQuadrant,       // E[((c * nzc + n) * ny + v) * nx + u] = the embedded kernel at (u, v), i.e. the
+                         // value at the offset (-u, -v); the rest mirrors it
+        kQuadrantPairs,  // the same as unevaluated FP32 pairs (float2)
+    };
+    Mode mode;
+    int px, py;              // kHalfRows
+    double factor[kMaxComp];  // value = factor[component] times the corner sum (upsilon for SI units)
+};
+// Output of the given mode in SI units.
+GenOut gen_out(GenOut::Mode mode, int px = 0, int py = 0);
+// Layers n0 .. n1 (nzc = n1 - n0), one slot per selected component.
+cudaError_t launch_kernel_gen(const Geometry& g, const GenOut& o, unsigned comps, int n0, int n1, void* out,
+                              cudaStream_t s);
 
 // ---- row transforms (fft_rows.cu) ----
 // Real rows -> half spectra, written transposed:
@@ -290,13 +305,18 @@ template <> cudaError_t launch_adjoint_columns<float>(int, const ColumnArgs&, co
                                                      const void*, int*, cudaStream_t, Batch);
 template <> cudaError_t launch_adjoint_columns<double>(int, const ColumnArgs&, const void*, const double*, void*,
                                                       const void*, int*, cudaStream_t, Batch);
-// Column FFT of embedded kernel row transforms and extraction of the stored
-// real numbers.  Ehat[kx][o][b] for b < py / 2 (row stride py / 2), o = c *
-// nzc + n; row py - b is row b times -1 for components odd in y (bit s of
-// oddv_mask), row py / 2 is zero.
-template <typename RO>
-cudaError_t launch_spec_extract(int log_n, const void* ehat, int kx_count, int nzc, int ncomp,
-                                int n0, int nz, int jp, unsigned imag_mask, unsigned oddv_mask, double scale,
-                                RO* spec, const void* tw64, int log_t, cudaStream_t s);
+
+// ---- kernel spectra of plane plans (spec_build.cu) ----
+struct SpecBuild {
+    int nx, ny, nz, ny2;  // ny2: ny rounded up to even, the row length of T
+    int ncomp, kx_count, jp, log_px, log_py;
+    unsigned oddu_mask, oddv_mask;  // bit s: component slot s is odd in x, in y
+};
+// Spectra of the layers n0 .. n0 + nzc from their quadrants E (kernel_gen;
+// doubles with fp64, else FP32 pairs).  T: staging, kx_count * ncomp * nzc *
+// ny2 values of 8 bytes.  factor: per slot, what the transform is multiplied
+// by (times 1 / (px py)).  tw: W_(2^log_t) in FP64 (fp64) or FP32 pairs.
+cudaError_t launch_spec_build_chunk(const SpecBuild& b, int fp64, const void* E, int nzc, int n0, void* T,
+                                    const double* factor, void* spec, const void* tw, int log_t, cudaStream_t s);
 
 }  // namespace grav

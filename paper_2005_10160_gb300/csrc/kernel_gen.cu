@@ -22,28 +22,47 @@
 //
 // One thread per offset (u, v) of the quadrant u, v >= 0, in tiles that
 // share their corner terms (see kernel_gen below).  Walking down the layers,
-// each thread writes the four mirrored offsets (+-u, +-v) using the
-// component's parity under reflection (Sec. 2.2), so the stored kernel is
-// exactly even or odd.
+// each thread writes its quadrant value, or the four mirrored offsets
+// (+-u, +-v) using the component's parity under reflection (Sec. 2.2), so the
+// kernel is exactly even or odd.
+#include <algorithm>
+
+#include "corner_terms.cuh"
 #include "grav_internal.h"
 
 namespace grav {
 
 namespace {
 
+// asinh(v / rho), inv = 1 / rho > 0, s = rho + sqrt(rho^2 + v^2), by
+// asinh(q) = log1p(q + q^2 / (1 + sqrt(1 + q^2))), which keeps the relative
+// accuracy of small q.
+__device__ __forceinline__ double asinh_ratio(double v, double inv, double s, const CornerTables& t) {
+    const double a = fabs(v), q = a * inv;
+    return copysign(log1p_pos(fma(q, a / s, q), t), v);
+}
+
+// A distance and its inverse.
+struct Dist { double d, inv; };
+__device__ __forceinline__ Dist distance(double a, double b) {
+    const double d = sqrt(a * a + b * b);
+    return Dist{d, 1.0 / d};
+}
+
 // NC: components kept per corner, 7 (gz ... gzz) or 9 (with gx, gy); plans
-// without gx, gy use 7 so that the kernel keeps fewer registers.
+// without gx, gy use 7 so that the kernel keeps fewer registers.  rxy, rxz,
+// ryz: distances in the coordinate planes.
 template <int NC>
-__device__ __forceinline__ void corner_terms(double x, double y, double z, unsigned comps, double (&F)[NC]) {
-    const double x2 = x * x, y2 = y * y, z2 = z * z;
-    const double r = sqrt(x2 + y2 + z2);
+__device__ __forceinline__ void corner_terms(double x, double y, double z, double r, Dist rxy, Dist rxz, Dist ryz,
+                                             unsigned comps, const CornerTables& t, double (&F)[NC]) {
     double ay = 0.0, ax = 0.0, az = 0.0, tz = 0.0, tx = 0.0, ty = 0.0;
-    if (comps & (GRAV_GZ | GRAV_GXZ | GRAV_GX)) ay = asinh(y / sqrt(x2 + z2));
-    if (comps & (GRAV_GZ | GRAV_GYZ | GRAV_GY)) ax = asinh(x / sqrt(y2 + z2));
-    if (comps & (GRAV_GXY | GRAV_GX | GRAV_GY)) az = asinh(z / sqrt(x2 + y2));
-    if (comps & (GRAV_GZ | GRAV_GZZ)) tz = atan(x * y / (z * r));
-    if (comps & (GRAV_GXX | GRAV_GX)) tx = atan(y * z / (x * r));
-    if (comps & (GRAV_GYY | GRAV_GY)) ty = atan(x * z / (y * r));
+    const double xa = fabs(x), ya = fabs(y), za = fabs(z);
+    if (comps & (GRAV_GZ | GRAV_GXZ | GRAV_GX)) ay = asinh_ratio(y, rxz.inv, r + rxz.d, t);
+    if (comps & (GRAV_GZ | GRAV_GYZ | GRAV_GY)) ax = asinh_ratio(x, ryz.inv, r + ryz.d, t);
+    if (comps & (GRAV_GXY | GRAV_GX | GRAV_GY)) az = asinh_ratio(z, rxy.inv, r + rxy.d, t);
+    if (comps & (GRAV_GZ | GRAV_GZZ)) tz = copysign(atan_ratio(xa * ya, za * r, t), x * y * z);
+    if (comps & (GRAV_GXX | GRAV_GX)) tx = copysign(atan_ratio(ya * za, xa * r, t), x * y * z);
+    if (comps & (GRAV_GYY | GRAV_GY)) ty = copysign(atan_ratio(xa * za, ya * r, t), x * y * z);
     F[0] = -(x * ay + y * ax - z * tz);
     F[1] = tx;
     F[2] = -az;
@@ -57,102 +76,157 @@ __device__ __forceinline__ void corner_terms(double x, double y, double z, unsig
     }
 }
 
+// v as an unevaluated FP32 pair; the high part truncates v by integer
+// arithmetic (conversions run at the FP64 rate), 0 below FP32's range.
+__device__ __forceinline__ float2 split_pair(double v) {
+    const uint64_t b = bits_of(v);
+    const int e = (int)((b >> 52) & 0x7ff) - 1023 + 127;
+    const bool ok = e > 0 && e < 255;
+    const uint32_t hb = (uint32_t)(b >> 63) << 31 | (uint32_t)(e & 255) << 23 | (uint32_t)((b >> 29) & 0x7fffffu);
+    const double hd = of_bits(b & ~0x1fffffffull);
+    return ok ? make_float2(__uint_as_float(hb), (float)(v - hd)) : make_float2((float)v, 0.f);
+}
+
 // Offsets per CTA: a kGenTX x kGenTY tile of the quadrant.  Neighbouring
 // offsets share prism corners (the far x-corner of offset u is the near one
 // of u + 1), so the CTA evaluates the corner terms of its (kGenTX + 1) x
-// (kGenTY + 1) corners once per z-level into shared memory (two levels kept:
-// the bottom of layer n is the top of layer n + 1) and every thread forms
-// its offset's kernel values from its eight corners.  The FP64 work per
-// offset and level drops from four corner evaluations to about 1.2.
-constexpr int kGenTX = 32, kGenTY = 8;
+// (kGenTY + 1) corners once per z-level, keeps the difference to the level
+// above in shared memory, and every thread forms its offsets' kernel values
+// from four differences.  blockIdx.z takes a run of `per` layers.
+//
+// Bound by FP64 issue.  512 x 512 x 64, six components: 14.7 ms with the
+// library's asinh and atan, tiles of 32 x 8 and one run of layers.
+constexpr int kGenTX = 32, kGenTY = 16, kGenThreads = 256;
+constexpr int kGenCX = kGenTX + 1, kGenCY = kGenTY + 1, kGenCor = kGenCX * kGenCY;
+constexpr size_t gen_smem(int nc) {
+    return sizeof(CornerTables) + (size_t)kGenCor * 2 * nc * sizeof(double) +
+           (size_t)(kGenCor + kGenCX + kGenCY) * sizeof(Dist);
+}
 
 template <int NC>
-__global__ void __launch_bounds__(kGenTX * kGenTY)
-    kernel_gen(Geometry g, unsigned comps, int n0, int n1, int mode, int px, int py, double* __restrict__ out) {
-    constexpr int CX = kGenTX + 1, CY = kGenTY + 1, NCOR = CX * CY, NT = kGenTX * kGenTY;
-    __shared__ double F[2][CY][CX][NC];  // corner terms of two z-levels
-    const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * kGenTX + tx;
+__global__ void __launch_bounds__(kGenThreads)
+    kernel_gen(Geometry g, GenOut o, unsigned comps, int n0, int n1, int per, void* __restrict__ out) {
+    constexpr int CX = kGenCX, NT = kGenThreads;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    CornerTables& tab = *reinterpret_cast<CornerTables*>(smem_raw);
+    double* F = reinterpret_cast<double*>(smem_raw + sizeof(CornerTables));  // corner terms of the level above
+    double* D = F + kGenCor * NC;   // level minus the level above
+    Dist* rxy = reinterpret_cast<Dist*>(D + kGenCor * NC);  // sqrt(x^2 + y^2) per corner
+    Dist* rxz = rxy + kGenCor;                              // sqrt(x^2 + z^2), sqrt(y^2 + z^2) of the level
+    Dist* ryz = rxz + CX;
+    const int tid = threadIdx.x, tx = tid % kGenTX, ty0 = tid / kGenTX;
     const int u0 = blockIdx.x * kGenTX, v0 = blockIdx.y * kGenTY;
-    const int u = u0 + tx, v = v0 + ty;
+    const int u = u0 + tx;
+    const int first = n0 + blockIdx.z * per, last = min(n1, first + per);
 
-    // corner terms of z-level z into buffer buf: corner (cu, cv) sits at
-    // x = (1/2 - cu) dx, y = (1/2 - cv) dy (station at the origin)
-    auto level = [&](int buf, double z) {
-        for (int e = tid; e < NCOR; e += NT) {
+    // corner (cx, cy) sits at x = (1/2 - u0 - cx) dx, y = (1/2 - v0 - cy) dy (station at the origin)
+    auto cx_of = [&](int cx) { return (0.5 - (u0 + cx)) * g.dx; };
+    auto cy_of = [&](int cy) { return (0.5 - (v0 + cy)) * g.dy; };
+    for (int e = tid; e < CornerTables::LOGS; e += NT) corner_table_entry(tab, e);
+    for (int e = tid; e < kGenCor; e += NT) {
+        rxy[e] = distance(cx_of(e % CX), cy_of(e / CX));
+    }
+    // corner terms of z-level z into F and, but for the first level, their change into D
+    auto level = [&](double z, bool difference) {
+        if (tid < CX) rxz[tid] = distance(cx_of(tid), z);
+        else if (tid >= 64 && tid < 64 + kGenCY) ryz[tid - 64] = distance(cy_of(tid - 64), z);
+        __syncthreads();  // distances in place; D and the tables free or in place
+        for (int e = tid; e < kGenCor; e += NT) {
             const int cy = e / CX, cx = e - cy * CX;
-            const int cu = u0 + cx, cv = v0 + cy;
+            if (u0 + cx > g.nx || v0 + cy > g.ny) continue;
             double t[NC];
-            if (cu <= g.nx && cv <= g.ny) {
-                corner_terms<NC>((0.5 - cu) * g.dx, (0.5 - cv) * g.dy, z, comps, t);
-            } else {
+            const double x = cx_of(cx), y = cy_of(cy);
+            corner_terms<NC>(x, y, z, sqrt(x * x + y * y + z * z), rxy[e], rxz[cx], ryz[cy], comps, tab, t);
 #pragma unroll
-                for (int c = 0; c < NC; ++c) t[c] = 0.0;
+            for (int c = 0; c < NC; ++c) {
+                if (!(comps & (1u << c))) continue;
+                if (difference) D[e * NC + c] = t[c] - F[e * NC + c];
+                F[e * NC + c] = t[c];
             }
-#pragma unroll
-            for (int c = 0; c < NC; ++c) F[buf][cy][cx][c] = t[c];
         }
+        __syncthreads();
     };
 
     const int nzc = n1 - n0;
     const int wx = 2 * g.nx - 1, wy = 2 * g.ny - 1;
-    int cur = 0;
-    level(cur, -g.h - n0 * g.dz);
-    for (int n = n0; n < n1; ++n) {
-        level(cur ^ 1, -g.h - (n + 1) * g.dz);
-        __syncthreads();
-        if (u < g.nx && v < g.ny) {
+    level(-g.h - first * g.dz, false);
+    for (int n = first; n < last; ++n) {
+        level(-g.h - (n + 1) * g.dz, true);
+        for (int ty = ty0; ty < kGenTY; ty += NT / kGenTX) {
+            const int v = v0 + ty;
+            if (u >= g.nx || v >= g.ny) continue;
 #pragma unroll
             for (int c = 0; c < NC; ++c) {
                 if (!(comps & (1u << c))) continue;
                 const int s = __popc(comps & ((1u << c) - 1u));  // output slot of component c
                 // mu_ijk: +1 for the bottom z-level when i + j is even; corners
                 // (u + i, v + j)
-                const double d00 = F[cur ^ 1][ty][tx][c] - F[cur][ty][tx][c];
-                const double d01 = F[cur ^ 1][ty + 1][tx][c] - F[cur][ty + 1][tx][c];
-                const double d10 = F[cur ^ 1][ty][tx + 1][c] - F[cur][ty][tx + 1][c];
-                const double d11 = F[cur ^ 1][ty + 1][tx + 1][c] - F[cur][ty + 1][tx + 1][c];
-                const double K = kUpsilon * ((d00 - d01) - (d10 - d11));
+                const double* d = D + (ty * CX + tx) * NC + c;
+                const double K = o.factor[c] * ((d[0] - d[CX * NC]) - (d[NC] - d[CX * NC + NC]));
+                const bool zero = (u == 0 && odd_u(c)) || (v == 0 && odd_v(c));
+                if (o.mode == GenOut::kQuadrant || o.mode == GenOut::kQuadrantPairs) {
+                    // the offset (-u, -v)
+                    const double val = zero ? 0.0 : odd_u(c) != odd_v(c) ? -K : K;
+                    const size_t idx = (((size_t)s * nzc + (n - n0)) * g.ny + v) * g.nx + u;
+                    if (o.mode == GenOut::kQuadrant) static_cast<double*>(out)[idx] = val;
+                    else static_cast<float2*>(out)[idx] = split_pair(val);
+                    continue;
+                }
+                double* dst = static_cast<double*>(out);
                 for (int mu = 0; mu < (u > 0 ? 2 : 1); ++mu) {
                     for (int mv = 0; mv < (v > 0 ? 2 : 1); ++mv) {
                         double val = K;
                         if (mu && odd_u(c)) val = -val;
                         if (mv && odd_v(c)) val = -val;
-                        if ((u == 0 && odd_u(c)) || (v == 0 && odd_v(c))) val = 0.0;
+                        if (zero) val = 0.0;
                         const int U = mu ? -u : u, V = mv ? -v : v;
-                        size_t idx;
-                        if (mode == 0) {
-                            const int a = (px - U) & (px - 1), b = (py - V) & (py - 1);
-                            idx = (((size_t)s * nzc + (n - n0)) * py + b) * px + a;
-                        } else if (mode == 2) {
+                        if (o.mode == GenOut::kHalfRows) {
                             // rows b = -V < py / 2 only (V <= 0): the rest mirror them
                             if (V > 0) continue;
-                            const int a = (px - U) & (px - 1), b = -V;
-                            idx = (((size_t)s * nzc + (n - n0)) * (py / 2) + b) * px + a;
+                            const int a = (o.px - U) & (o.px - 1), b = -V;
+                            dst[(((size_t)s * nzc + (n - n0)) * (o.py / 2) + b) * o.px + a] = val;
                         } else {
-                            idx = (((size_t)s * g.nz + n) * wy + (V + g.ny - 1)) * wx + (U + g.nx - 1);
+                            dst[(((size_t)s * g.nz + n) * wy + (V + g.ny - 1)) * wx + (U + g.nx - 1)] = val;
                         }
-                        out[idx] = val;
                     }
                 }
             }
         }
-        __syncthreads();  // the next level overwrites this level's top buffer
-        cur ^= 1;
     }
+}
+
+template <int NC>
+cudaError_t gen_launch(const Geometry& g, const GenOut& o, unsigned comps, int n0, int n1, void* out, cudaStream_t s) {
+    constexpr auto k = kernel_gen<NC>;
+    cudaError_t e = ensure_smem_limit<k>();
+    if (e != cudaSuccess) return e;
+    dim3 grid((g.nx + kGenTX - 1) / kGenTX, (g.ny + kGenTY - 1) / kGenTY);
+    // runs of layers: each costs one level more, so at least 8 layers, and no
+    // more runs than give every SM 12 CTAs
+    const int nz = n1 - n0, tiles = (int)(grid.x * grid.y);
+    const int want = std::max(1, std::min((12 * 152 + tiles - 1) / tiles, nz / 8));
+    const int per = (nz + want - 1) / want;
+    grid.z = (nz + per - 1) / per;
+    k<<<grid, kGenThreads, gen_smem(NC), s>>>(g, o, comps, n0, n1, per, out);
+    return cudaGetLastError();
 }
 
 }  // namespace
 
-cudaError_t launch_kernel_gen(const Geometry& g, unsigned comps, int n0, int n1, int mode, int px, int py,
-                              double* out, cudaStream_t s) {
-    const dim3 block(kGenTX, kGenTY);
-    const dim3 grid((g.nx + kGenTX - 1) / kGenTX, (g.ny + kGenTY - 1) / kGenTY);
+cudaError_t launch_kernel_gen(const Geometry& g, const GenOut& o, unsigned comps, int n0, int n1, void* out,
+                              cudaStream_t s) {
     comps &= kCompBits;
-    if (comps & (GRAV_GX | GRAV_GY))
-        kernel_gen<9><<<grid, block, 0, s>>>(g, comps, n0, n1, mode, px, py, out);
-    else
-        kernel_gen<7><<<grid, block, 0, s>>>(g, comps, n0, n1, mode, px, py, out);
-    return cudaGetLastError();
+    return comps & (GRAV_GX | GRAV_GY) ? gen_launch<9>(g, o, comps, n0, n1, out, s)
+                                       : gen_launch<7>(g, o, comps, n0, n1, out, s);
+}
+
+GenOut gen_out(GenOut::Mode mode, int px, int py) {
+    GenOut o{};
+    o.mode = mode;
+    o.px = px;
+    o.py = py;
+    for (double& f : o.factor) f = kUpsilon;
+    return o;
 }
 
 }  // namespace grav
