@@ -112,6 +112,52 @@ __global__ void __launch_bounds__(NT, 2) row_r2c_kernel(const R* __restrict__ in
     }
 }
 
+// FP64 rows of P = 2N points with at most N nonzero values (the row stage of
+// every FP64 plan): the even and the odd bins are two N-point transforms,
+//   Z(2k + p) = sum_{x < N} (z[x] W_P^(p x)) W_N^(x k),
+// with twiddles from per-pass tables.  FP64 issue bounds the stage, and this
+// form needs about 30 FP64 instructions a point where the P-point transform
+// with computed twiddle powers needs 42: 512 x 512 x 64, 1.51 ms before.
+template <int LOGN, int NSEQ, int NT>
+__global__ void __launch_bounds__(NT, 2) row_r2c_half_kernel(const double* __restrict__ in, size_t in_ostride,
+                                                           size_t in_istride, int l_in, int I, int O,
+                                                           double2* __restrict__ out, int i_pad,
+                                                           const double2* __restrict__ tw, int shift_n, int shift_p,
+                                                           size_t in_bstride, size_t out_bstride) {
+    using C = double2;
+    constexpr int N = 1 << LOGN, SSTR = seq_stride<C>(N);
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    C* buf = reinterpret_cast<C*>(smem_raw);  // bins of (row pair s, parity p) at sequence 2 s + p
+    C* tab = buf + 2 * NSEQ * SSTR;
+    const int tid = threadIdx.x;
+    const int o = blockIdx.y, i_base = blockIdx.x * (2 * NSEQ);
+    out += blockIdx.z * out_bstride;
+    const double* in_o = in + blockIdx.z * in_bstride + (size_t)o * in_ostride;
+    build_tw_tab<C, LOGN, NT>(tab, tw, shift_n, tid);
+    __syncthreads();
+    block_fft_tab_from<C, LOGN, 2 * NSEQ, NT, false>(buf, SSTR, tab, tid, [&](int sq, int m) {
+        const int i0 = i_base + 2 * (sq >> 1);
+        C v = cmk<C>(0, 0);
+        if (m < l_in) {
+            if (i0 < I) v.x = in_o[(size_t)i0 * in_istride + m];
+            if (i0 + 1 < I) v.y = in_o[(size_t)(i0 + 1) * in_istride + m];
+            if (sq & 1) v = cmul(v, tw[m << shift_p]);
+        }
+        return v;
+    });
+    for (int e = tid; e < NSEQ * (N + 1); e += NT) {
+        const int s = e % NSEQ, kx = e / NSEQ, q = kx & 1, k = kx >> 1;
+        const int i0 = i_base + 2 * s, i1 = i0 + 1;
+        if (i0 >= I) continue;
+        const C* z = buf + (2 * s + q) * SSTR;  // kx and P - kx have the same parity
+        const C zk = z[sidx<C>(k)], zm = cconj(z[sidx<C>(q ? N - 1 - k : (N - k) & (N - 1))]);
+        const C d = csub(zk, zm);
+        C* dst = out + ((size_t)kx * O + o) * i_pad + i0;
+        dst[0] = cmk<C>(0.5 * (zk.x + zm.x), 0.5 * (zk.y + zm.y));
+        if (i1 < I) dst[1] = cmk<C>(0.5 * d.y, -0.5 * d.x);
+    }
+}
+
 // FP32 rows of length P = 2048 with at most 1024 nonzero values (the row
 // stages of every mesh with 513 <= nx <= 1024): the even and the odd outputs
 // are two independent 1024-point transforms,
@@ -487,6 +533,20 @@ inline int sm_count() {
     return n;
 }
 
+template <int LOGP>
+cudaError_t r2c_half_launch(const double* in, size_t in_ostride, size_t in_istride, int l_in, int I, int O, void* out,
+                            int i_pad, const void* tw, int log_t, cudaStream_t s, Batch b) {
+    constexpr int NSEQ = nseq_for<double>(LOGP), NT = 512, LOGN = LOGP - 1;
+    constexpr size_t smem = ((size_t)2 * NSEQ * seq_stride<double2>(1 << LOGN) + tw_tab_len(LOGN)) * sizeof(double2);
+    constexpr auto k = row_r2c_half_kernel<LOGN, NSEQ, NT>;
+    cudaError_t e = ensure_smem_limit<k>();
+    if (e != cudaSuccess) return e;
+    dim3 grid((I + 2 * NSEQ - 1) / (2 * NSEQ), O, b.count);
+    k<<<grid, NT, smem, s>>>(in, in_ostride, in_istride, l_in, I, O, (double2*)out, i_pad, (const double2*)tw,
+                             log_t - LOGN, log_t - LOGP, b.in, b.out);
+    return cudaGetLastError();
+}
+
 template <typename R, int LOGP>
 cudaError_t r2c_impl(const R* in, size_t in_ostride, size_t in_istride, int l_in, int I, int O, void* out, int i_pad,
                      const void* tw, int log_t, cudaStream_t s, Batch b, int* err) {
@@ -521,6 +581,8 @@ cudaError_t r2c_impl(const R* in, size_t in_ostride, size_t in_istride, int l_in
         if (vec) return r2c_launch<R, LOGP, true>(in, in_ostride, in_istride, l_in, I, O, out, i_pad, tw, log_t, s, b);
         return r2c_launch<R, LOGP, false>(in, in_ostride, in_istride, l_in, I, O, out, i_pad, tw, log_t, s, b);
     } else {
+        if (l_in <= (1 << LOGP) / 2)
+            return r2c_half_launch<LOGP>(in, in_ostride, in_istride, l_in, I, O, out, i_pad, tw, log_t, s, b);
         return r2c_launch<R, LOGP, false>(in, in_ostride, in_istride, l_in, I, O, out, i_pad, tw, log_t, s, b);
     }
 }

@@ -199,11 +199,18 @@ __global__ void __launch_bounds__(ColShape<LOGN>::J, ColShape<LOGN>::J <= 256 ? 
                 return v;
             });
         }
-        R part[NC][4];
+        // FP32: the round's terms, which enter the compensated sum as one; FP64:
+        // straight into the sum (an add per round and value would be an eighth
+        // of the kernel's FP64 instructions)
+        R round[KAHAN ? NC : 1][4];
+        R(*part)[4] = acc;
+        if constexpr (KAHAN) {
 #pragma unroll
-        for (int c = 0; c < NC; ++c)
+            for (int c = 0; c < NC; ++c)
 #pragma unroll
-            for (int j = 0; j < 4; ++j) part[c][j] = 0;
+                for (int j = 0; j < 4; ++j) round[c][j] = 0;
+            part = round;
+        }
         if (!nyq) {
 #pragma unroll
             for (int l = 0; l < NSEQ; ++l) {
@@ -236,13 +243,12 @@ __global__ void __launch_bounds__(ColShape<LOGN>::J, ColShape<LOGN>::J <= 256 ? 
                 }
             }
         }
+        if constexpr (KAHAN) {
 #pragma unroll
-        for (int c = 0; c < NC; ++c)
+            for (int c = 0; c < NC; ++c)
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                if (KAHAN) kahan_add(acc[c][j], cmp[c][j], part[c][j]);
-                else acc[c][j] += part[c][j];
-            }
+                for (int j = 0; j < 4; ++j) kahan_add(acc[c][j], cmp[c][j], part[c][j]);
+        }
         __syncthreads();  // stages and FFT buffers free again
         if (tid == 0) {
             fence_proxy_async_smem();
@@ -443,9 +449,17 @@ FwdSmem forward_smem(int log_n, int ny_pad, int ncomp, int jp, int max_bytes) {
     L.stage_bytes = (L.x_bytes + L.s_bytes + 127u) & ~127u;
     const uint32_t fft_bytes = (uint32_t)(NSEQ * spad_len<C>(1 << log_n) * sizeof(C));
     const uint32_t tw_bytes = (uint32_t)(((1u << log_n) + tw_tab_len(log_n)) * sizeof(C));  // fold + pass tables
-    int depth = 2 * NSEQ;
-    while (depth >= NSEQ && (size_t)depth * L.stage_bytes + fft_bytes + tw_bytes + depth * 8 + 128 > (size_t)max_bytes)
-        --depth;
+    // CTAs of at most 256 threads: two per SM if NSEQ stages fit in half the
+    // shared memory (512 x 512 x 64 FP64, six components: a ring of 4 left one
+    // CTA of 8 warps per SM and the FP64 pipe 30% idle); else the deepest ring
+    // of one CTA.
+    auto deepest = [&](size_t limit) {
+        int d = 2 * NSEQ;
+        while (d >= NSEQ && (size_t)d * L.stage_bytes + fft_bytes + tw_bytes + d * 8 + 128 > limit) --d;
+        return d;
+    };
+    int depth = (1 << log_n) / 2 <= 256 ? deepest((size_t)max_bytes / 2 - 1024) : 0;
+    if (depth < NSEQ) depth = deepest((size_t)max_bytes);
     if (depth < NSEQ) return FwdSmem{};
     L.depth = depth;
     L.fft_off = depth * L.stage_bytes;
