@@ -66,8 +66,14 @@ __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.comm
 // Wait until every committed bulk store of this thread has read its shared
 // memory source (the buffer may then be rewritten).
 __device__ __forceinline__ void bulk_wait_read_all() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
-// Wait until every committed bulk store of this thread has completed.
-__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
+
+// Two floats from read-only global memory, loaded where the call stands: the compiler may move a plain load down to its use, which undoes a
+// look-ahead in registers.
+__device__ __forceinline__ float2 load_here2(const float* p) {
+    float2 v;
+    asm volatile("ld.global.nc.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+    return v;
+}
 
 // Per-thread asynchronous copy of 8 bytes global -> shared (both 8-byte
 // aligned); with valid = false nothing is read and the destination is

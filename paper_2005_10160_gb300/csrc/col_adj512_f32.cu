@@ -4,7 +4,7 @@
 // with both ky parities in one CTA and every warp transform doing the two
 // parities at once (warp_fft512x2).
 //
-// The layout is that of the 1024-point adjoint kernel (spectral_adj_wf.cuh):
+// The roles are those of the 1024-point adjoint kernel (spectral_adj_wf.cuh):
 // 24 warps at 80 registers.  Warps 16-23 first transform the residual
 // columns (component c in warp c, both parities) into slots 0 .. NC-1; thread
 // q of warps 0-15 keeps both bins of mirror pair q % 256 of parity q / 256

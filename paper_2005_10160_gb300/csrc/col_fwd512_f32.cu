@@ -2,7 +2,7 @@
 // 257 <= ny <= 512): both ky parities of a kx column in one CTA, each warp
 // transform doing the two parities of one layer at once.
 //
-// The layout is that of the 1024-point kernel (spectral_wf.cuh): 24 warps at
+// The roles are those of the 1024-point kernel (spectral_wf.cuh): 24 warps at
 // 80 registers, warps 0-15 accumulate (thread q: parity q / 256, mirror pair
 // q % 256, every component), warps 16-23 transform layers f, f + 8, ... from
 // their own X slot, which they refill by bulk copy.  A layer's F slot holds

@@ -3,18 +3,26 @@
 //   Z_n = IFFT_y( sum_c conj(S_c,n) . FFT_y(R_c) )
 // on one kx column and one ky parity (the same parity split as the forward).
 //
-// 24 warps at 80 registers a thread.  Warps 16-23 first transform the
+// 16 warps at 128 registers a thread.  Warps 8-15 first transform the
 // residual's row-transform columns (component f in warp f), one warp each,
-// in registers (warp_fft1024); thread q of warps 0-15 keeps both bins of
-// mirror pair q of every component in registers.  Then, layer by layer, the
-// combine threads form the layer's spectrum from their bins and the layer's
-// spectra values (read from global memory one layer ahead, after a bulk L2
+// in registers (warp_fft1024); thread t of warps 0-7 keeps both bins of the
+// mirror pairs 2t and 2t + 1 of every component in registers, with -i for
+// imaginary spectra and the mirror sign for odd components applied.  Then,
+// layer by layer, the combine threads form the layer's spectrum from their
+// bins and the layer's spectra values, as two-wide FP32 operations over the
+// two pairs (spectra read from global memory two layers ahead, after a bulk L2
 // prefetch eight layers ahead: the combine threads run ahead of the
 // transforms, so a load from DRAM would stall every layer) and write it
 // into a ring slot; FFT warp f inverse-transforms layers f, f + 8, ... from
 // the slot (which is also its transpose area) and writes the rows y < ny.
 // The combine threads run up to (ring depth - 8) layers ahead of the
-// transforms.  Every wait is bounded.
+// transforms.  The FFT warps form the Nyquist bin themselves.  Every wait is
+// bounded.
+//
+// 1024 x 1024 x 100, six components: 760 us (4.2 GB: 5.5 TB/s); 993 with one
+// pair a thread (24 warps at 80 registers, spectra one layer ahead), 949 with
+// two pairs while the compiler moved the spectra loads down to their use and
+// the residual columns were read after the tables.
 #pragma once
 #include "async_copy.cuh"
 #include "grav_internal.h"
@@ -26,11 +34,11 @@ namespace grav {
 
 struct AwShape {
     static constexpr int N = 1024;
-    static constexpr int J = 512;     // combine threads (16 warps), one mirror pair each
+    static constexpr int J = 512;     // mirror pairs
+    static constexpr int MT = J / 2;  // combine threads (8 warps), two pairs each
     static constexpr int FWARPS = 8;  // FFT warps
-    static constexpr int NT = J + 32 * FWARPS;
+    static constexpr int NT = MT + 32 * FWARPS;
     static constexpr int SLOT = kWarpFftSlot;
-    static constexpr int REGS = 80;
     static constexpr int JP = 516;    // spectra row pitch: J + 1 rounded up to 4
     static constexpr int PF = 8;      // spectra prefetch distance into L2 (layers)
 };
@@ -40,17 +48,13 @@ struct AwSmem {
     uint32_t slot_off, tw_off, t2_off, stage_off, bar_off, flag_off, total;
 };
 
-// IM, OV: the plan's imaginary-spectrum and odd-in-y component masks when
-// known at compile time (the all-six-components request), else kRuntimeMask.
-constexpr unsigned kRuntimeMask = ~0u;
-
-template <int NC, unsigned IM = kRuntimeMask, unsigned OV = kRuntimeMask>
-__global__ void __maxnreg__(AwShape::REGS)
+template <int NC>
+__global__ void __launch_bounds__(AwShape::NT, 1)
     adjoint_column_wf_kernel(ColumnArgs a, AwSmem L, const float2* __restrict__ Xr, const float* __restrict__ spec,
                              float2* __restrict__ Z, const float2* __restrict__ tw, int* __restrict__ err,
                              size_t x_bstride, size_t z_bstride, const __grid_constant__ CUtensorMap zmap) {
     using C = float2;
-    constexpr int N = AwShape::N, J = AwShape::J, FW = AwShape::FWARPS, NT = AwShape::NT;
+    constexpr int N = AwShape::N, J = AwShape::J, MT = AwShape::MT, FW = AwShape::FWARPS, NT = AwShape::NT;
     constexpr int FS = AwShape::SLOT, JP = AwShape::JP, S_ROW = NC * JP;
     static_assert(NC <= FW, "one residual transform per FFT warp");
     extern __shared__ __align__(128) unsigned char smem[];
@@ -69,9 +73,24 @@ __global__ void __maxnreg__(AwShape::REGS)
     Z += blockIdx.y * z_bstride;
     const float* Sk = request_spec(a, spec, blockIdx.y) + (size_t)(r * a.kx_count + kx) * nz * S_ROW;
 
+    // FFT warp c reads component c's residual column while the tables are built
+    const bool transforms = warp >= MT / 32 && warp - MT / 32 < NC;
+    float2 u[32];
+    if (transforms) {
+        const C* col = Xr + ((size_t)kx * a.ncomp + (warp - MT / 32)) * a.ny_pad;
+#pragma unroll
+        for (int n1 = 0; n1 < 32; ++n1) {
+            const int m = 32 * n1 + lane;
+            u[n1] = m < ny ? col[m] : make_float2(0.f, 0.f);
+        }
+    }
     if (tid == 0) {
+        // spectra of the first PF layers into L2, later one layer more each
+        // iteration, so that the loads ahead hit L2
+        for (int n = 0; n < AwShape::PF && n < nz; ++n)
+            bulk_prefetch_l2(Sk + (size_t)n * S_ROW, S_ROW * sizeof(float));
         for (int s = 0; s < L.dz; ++s) {
-            mbar_init(&zfull[s], J);
+            mbar_init(&zfull[s], MT);
             mbar_init(&zempty[s], 32);
         }
         *abort = 0;
@@ -85,19 +104,11 @@ __global__ void __maxnreg__(AwShape::REGS)
     __syncthreads();
 
     // FFT_y of every component's residual column, into slots 0 .. NC-1
-    if (warp >= J / 32 && warp - J / 32 < NC) {
-        const int c = warp - J / 32;
-        const C* col = Xr + ((size_t)kx * a.ncomp + c) * a.ny_pad;
-        float2 u[32];
+    if (transforms) {
+        const int c = warp - MT / 32;
+        if (r) {
 #pragma unroll
-        for (int n1 = 0; n1 < 32; ++n1) {
-            const int m = 32 * n1 + lane;
-            C v = make_float2(0.f, 0.f);
-            if (m < ny) {
-                v = col[m];
-                if (r) v = cmul(v, tws[m]);  // fold for ky parity r
-            }
-            u[n1] = v;
+            for (int n1 = 0; n1 < 32; ++n1) u[n1] = cmul(u[n1], tws[32 * n1 + lane]);  // fold for ky parity r
         }
         C* fb = ring + c * FS;
         warp_fft1024<false>(u, fb, t2, lane);
@@ -107,71 +118,74 @@ __global__ void __maxnreg__(AwShape::REGS)
     __syncthreads();
 
     bool failed = false;
-    if (tid < J) {
-        // ---------------- combine: thread q owns mirror pair q ----------------
-        const int q = tid;
-        int k1, k2;
-        pair_pos<N>(q, r, k1, k2);
-        const bool nyq = r == 0 && q == 0;  // second bin is the Nyquist row, with spectra values of its own
-        C rc[NC][2];
+    if (tid < MT) {
+        // ---------------- combine: thread t owns mirror pairs 2t, 2t + 1 ----------------
+        const int q = 2 * tid;
+        // bins of the two pairs: k1 = q, q + 1; k2 = N - q, N - q - 1 (even ky;
+        // pair 0: the Nyquist bin N / 2) or N - 1 - q, N - 2 - q (odd ky)
+        const int k2a = r ? N - 1 - q : q ? N - q : N / 2, k2b = r ? N - 2 - q : N - 1 - q;
+        // (the FFT warps form the Nyquist bin, which has spectra values of its own)
+        // bins, two-wide over the pairs: re and im of bin 1, of bin 2; conj(S) v
+        // with S = s or i s: -i and the mirror sign are applied here
+        float2 rc[NC][4];
 #pragma unroll
         for (int c = 0; c < NC; ++c) {
-            rc[c][0] = ring[c * FS + k1];
-            rc[c][1] = ring[c * FS + k2];
+            const C* fb = ring + c * FS;
+            C a1 = fb[q], b1 = fb[q + 1], a2 = fb[k2a], b2 = fb[k2b];
+            if ((a.imag_mask >> c) & 1u) {
+                a1 = make_float2(a1.y, -a1.x);
+                b1 = make_float2(b1.y, -b1.x);
+                a2 = make_float2(a2.y, -a2.x);
+                b2 = make_float2(b2.y, -b2.x);
+            }
+            if ((a.oddv_mask >> c) & 1u) {
+                a2 = make_float2(-a2.x, -a2.y);
+                b2 = make_float2(-b2.x, -b2.y);
+            }
+            rc[c][0] = make_float2(a1.x, b1.x);
+            rc[c][1] = make_float2(a1.y, b1.y);
+            rc[c][2] = make_float2(a2.x, b2.x);
+            rc[c][3] = make_float2(a2.y, b2.y);
         }
-        const unsigned imag = IM == kRuntimeMask ? a.imag_mask : IM;
-        const unsigned oddv = OV == kRuntimeMask ? a.oddv_mask : OV;
         cta_sync();  // every combine thread has its bins: the slots become the ring
         const float* Sq = Sk + q;
-        float sv[NC], se[NC];
-        auto load = [&](int n) {
+        float2 sv[2][NC];
+        auto load = [&](int n, float2 (&s)[NC]) {
+            if (n >= nz) return;
             const float* row = Sq + (size_t)n * S_ROW;
 #pragma unroll
-            for (int c = 0; c < NC; ++c) {
-                sv[c] = __ldg(row + c * JP);
-                se[c] = nyq ? __ldg(row + c * JP + (J - q)) : 0.f;
-            }
+            for (int c = 0; c < NC; ++c) s[c] = load_here2(row + c * JP);
         };
-        // spectra of the first PF layers into L2 (thread 0), then one layer
-        // more each iteration, so that the one-layer-ahead loads hit L2
         constexpr int PF = AwShape::PF;
-        if (q == 0)
-            for (int n = 0; n < PF && n < nz; ++n) bulk_prefetch_l2(Sk + (size_t)n * S_ROW, S_ROW * sizeof(float));
-        if (nz > 0) load(0);
+        load(0, sv[0]);
+        load(1, sv[1]);
         int sz = 0, wrap = 0;  // ring slot of layer n (n % dz) and n / dz, stepped with n
-        for (int n = 0; n < nz; ++n) {
-            if (q == 0 && n + PF < nz) bulk_prefetch_l2(Sk + (size_t)(n + PF) * S_ROW, S_ROW * sizeof(float));
-            if (n >= L.dz && !ws_wait(&zempty[sz], (uint32_t)((wrap - 1) & 1), abort)) {
-                failed = true;
-                break;
-            }
-            C z1 = make_float2(0.f, 0.f), z2 = make_float2(0.f, 0.f);
+        auto layer = [&](int n, float2 (&s)[NC]) {
+            if (tid == 0 && n + PF < nz) bulk_prefetch_l2(Sk + (size_t)(n + PF) * S_ROW, S_ROW * sizeof(float));
+            if (n >= L.dz && !ws_wait(&zempty[sz], (uint32_t)((wrap - 1) & 1), abort)) return false;
+            float2 z[4];
 #pragma unroll
-            for (int c = 0; c < NC; ++c) {
-                const float s1 = sv[c];
-                const float s2 = nyq ? se[c] : (((oddv >> c) & 1u) ? -s1 : s1);
-                const C v1 = rc[c][0], v2 = rc[c][1];
-                // conj(S) v with S = s (real spectrum) or i s (imaginary spectrum)
-                if ((imag >> c) & 1u) {
-                    z1.x += s1 * v1.y;
-                    z1.y -= s1 * v1.x;
-                    z2.x += s2 * v2.y;
-                    z2.y -= s2 * v2.x;
-                } else {
-                    z1.x += s1 * v1.x;
-                    z1.y += s1 * v1.y;
-                    z2.x += s2 * v2.x;
-                    z2.y += s2 * v2.y;
-                }
-            }
-            if (n + 1 < nz) load(n + 1);
+            for (int j = 0; j < 4; ++j) z[j] = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int c = 0; c < NC; ++c)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) z[j] = __ffma2_rn(s[c], rc[c][j], z[j]);
+            load(n + 2, s);
             C* zb = ring + sz * FS;
-            zb[k1] = z1;
-            zb[k2] = z2;
+            *reinterpret_cast<float4*>(zb + q) = make_float4(z[0].x, z[1].x, z[0].y, z[1].y);
+            zb[k2a] = make_float2(z[2].x, z[3].x);
+            zb[k2b] = make_float2(z[2].y, z[3].y);
             mbar_arrive(&zfull[sz]);
             if (++sz == L.dz) {
                 sz = 0;
                 ++wrap;
+            }
+            return true;
+        };
+        for (int n = 0; n < nz; n += 2) {
+            if (!layer(n, sv[0]) || (n + 1 < nz && !layer(n + 1, sv[1]))) {
+                failed = true;
+                break;
             }
         }
         if (cta_sync_or(failed || *abort)) {
@@ -179,7 +193,18 @@ __global__ void __maxnreg__(AwShape::REGS)
         }
     } else {
         // ---------------- FFT warp f: inverse transforms of layers f, f + 8, ... ----------------
-        const int f = warp - J / 32;
+        const int f = warp - MT / 32;
+        // even ky: lane c holds the Nyquist bin of component c and reads its
+        // spectra values, one of its layers ahead; their products add up to
+        // bin N / 2 = 32 x 16 of the layer (register 16 of lane 0)
+        const bool nyq = r == 0 && lane < NC;
+        C rn = make_float2(0.f, 0.f);
+        if (nyq) {
+            rn = ring[lane * FS + N / 2];
+            if ((a.imag_mask >> lane) & 1u) rn = make_float2(rn.y, -rn.x);
+        }
+        const float* Sn = Sk + (nyq ? lane : 0) * JP + J;
+        float sn = nyq && f < nz ? __ldg(Sn + (size_t)f * S_ROW) : 0.f;
         cta_sync();
         // ring slot of layer n (n % dz) and the parity of n / dz, stepped with
         // n (n advances by FW < dz)
@@ -196,6 +221,16 @@ __global__ void __maxnreg__(AwShape::REGS)
             float2 u[32];
 #pragma unroll
             for (int n1 = 0; n1 < 32; ++n1) u[n1] = zb[32 * n1 + lane];
+            if (r == 0) {
+                C v = cscale(rn, sn);
+                sn = nyq && n + FW < nz ? __ldg(Sn + (size_t)(n + FW) * S_ROW) : 0.f;
+#pragma unroll
+                for (int o = 4; o; o >>= 1) {
+                    v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
+                    v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
+                }
+                if (lane == 0) u[16] = v;
+            }
             __syncwarp();
             warp_fft1024<true>(u, zb, t2, lane);
             if (a.z_tiled) {
@@ -242,7 +277,7 @@ __global__ void __maxnreg__(AwShape::REGS)
                 ++wrap;
             }
         }
-        if (a.z_tiled && lane == 0) bulk_wait_all();  // every tensor store has landed
+        if (a.z_tiled && lane == 0) bulk_wait_read_all();  // every tensor store has read its buffer
         cta_sync_or(failed || *abort);
     }
 }
