@@ -77,6 +77,8 @@ _lib = None
 def lib() -> ctypes.CDLL:
     """The loaded library (raises if it was never built)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is None:
             if not os.path.exists(LIB_PATH):
