@@ -67,11 +67,25 @@ __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.comm
 // memory source (the buffer may then be rewritten).
 __device__ __forceinline__ void bulk_wait_read_all() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 
-// Two floats from read-only global memory, loaded where the call stands: the compiler may move a plain load down to its use, which undoes a
+// One and two floats from read-only global memory, loaded where the call
+// stands: the compiler may move a plain load down to its use, which undoes a
 // look-ahead in registers.
+__device__ __forceinline__ float load_here(const float* p) {
+    float v;
+    asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
 __device__ __forceinline__ float2 load_here2(const float* p) {
     float2 v;
     asm volatile("ld.global.nc.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float2 load_here(const float2* p) { return load_here2(&p->x); }
+
+// Two complex values (16-byte aligned) past L1, where the call stands.
+__device__ __forceinline__ float4 load_here4_cg(const float2* p) {
+    float4 v;
+    asm volatile("ld.global.cg.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
     return v;
 }
 

@@ -6,9 +6,11 @@
 // A tile is 8 row pairs (4 for P = 2048) of one layer; warps of even index
 // run the even bins, warps of odd index the odd ones, so the fold of the odd
 // bins is a warp-uniform branch.  Tiles are walked by a grid that fills the
-// machine once, so the twiddle tables are built once per CTA.  Rows of any
-// length and alignment are read with scalar loads, each element by the two
-// warps that need it (the second read hits L1).
+// machine once, so the twiddle tables are built once per CTA, and the next
+// tile's loads are issued, into the registers that a finished transform frees,
+// before the tile is written.  Rows of any length and alignment are read with
+// scalar loads, each element by the two warps that need it (the second read
+// hits L1).
 //
 // The areas of the transforms start 1 complex value apart modulo 16 (2 for
 // P = 2048) and the pairs of a warp are chosen so that the 16 lanes of each
@@ -23,6 +25,7 @@
 #include <climits>
 #include <algorithm>
 
+#include "async_copy.cuh"
 #include "grav_internal.h"
 #include "group_fft.cuh"
 
@@ -79,27 +82,31 @@ __global__ void __launch_bounds__(RowGroup<N>::NT, RowGroup<N>::MINB)
     float2* area = areas + (2 * s + p) * S::AREA;
     const float2* t2 = tab + p * N;
 
+    float2 u[G::V];
+    auto load = [&](unsigned t) {  // this lane's share of tile t's rows
+        const unsigned rest = t / rbs;
+        const int bz = (int)(rest / (unsigned)O), o = (int)(rest - (unsigned)bz * (unsigned)O);
+        const int i0 = (int)(t - rest * rbs) * S::ROWS + 2 * s;
+        const bool ha = t < ntiles && i0 < I, hb = ha && i0 + 1 < I;
+        const float* ra = in + (ha ? bz * in_bstride + (size_t)o * in_ostride + (size_t)i0 * in_istride : 0);
+        const float* rb = hb ? ra + in_istride : ra;
+#pragma unroll
+        for (int n2 = 0; n2 < G::V; ++n2) {
+            const int x = q + G::L * n2;
+            u[n2].x = ha && x < l_in ? load_here(ra + x) : 0.f;
+            u[n2].y = hb && x < l_in ? load_here(rb + x) : 0.f;
+        }
+    };
+    load(blockIdx.x);
     for (unsigned t = blockIdx.x; t < ntiles; t += gridDim.x) {
         const unsigned rest = t / rbs;
         const int ib = (int)(t - rest * rbs) * S::ROWS;
         const int bz = (int)(rest / (unsigned)O), o = (int)(rest - (unsigned)bz * (unsigned)O);
-        {
-            const int i0 = ib + 2 * s;
-            const bool ha = i0 < I, hb = i0 + 1 < I;
-            const float* ra = in + bz * in_bstride + (size_t)o * in_ostride + (size_t)(ha ? i0 : 0) * in_istride;
-            const float* rb = hb ? ra + in_istride : ra;
-            float2 u[G::V];
+        if (p) fold_regs<N>(u);
+        group_fft<N, false>(u, area, t2, q);
 #pragma unroll
-            for (int n2 = 0; n2 < G::V; ++n2) {
-                const int x = q + G::L * n2;
-                u[n2].x = ha && x < l_in ? __ldg(ra + x) : 0.f;
-                u[n2].y = hb && x < l_in ? __ldg(rb + x) : 0.f;
-            }
-            if (p) fold_regs<N>(u);
-            group_fft<N, false>(u, area, t2, q);
-#pragma unroll
-            for (int e = 0; e < G::V; ++e) area[group_bin<N>(q, e)] = u[e];
-        }
+        for (int e = 0; e < G::V; ++e) area[group_bin<N>(q, e)] = u[e];
+        if (t + gridDim.x < ntiles) load(t + gridDim.x);  // in flight while this tile is written
         __syncthreads();
         // A(kx) = (Z(kx) + conj Z(P - kx)) / 2, B(kx) = (Z(kx) - conj Z(P - kx)) / (2i);
         // kx = 2k + r and P - kx have the same parity r
@@ -130,14 +137,18 @@ __global__ void __launch_bounds__(RowGroup<N>::NT, RowGroup<N>::MINB)
 
 // Half spectra (in0, or in0 + in1) -> real rows, the first l_out values kept
 // (see launch_row_c2r): Z = A + i B is gathered into the even- and odd-bin
-// areas, two N-point inverse transforms, their unfolded sum stored.
-template <int N>
+// areas, two N-point inverse transforms, their unfolded sum stored.  AHEAD
+// (one input, N >= 512, where a CTA has several tiles): the next tile is read
+// into the registers that the transform has just freed, so that it arrives
+// while this tile is stored (512 x 512 x 64 adjoint: 89 -> 72 us).
+template <int N, bool AHEAD>
 __global__ void __launch_bounds__(RowGroup<N>::NT, RowGroup<N>::MINB)
     row_c2r_group_kernel(const float2* __restrict__ in0, const float2* __restrict__ in1, int I, int O, int i_pad,
                          float* __restrict__ out, size_t out_stride, int l_out, const float2* __restrict__ tw,
                          int shift_p, size_t in_bstride, size_t out_bstride, unsigned ntiles, unsigned rbs) {
     using S = RowGroup<N>;
     using G = GroupFft<N>;
+    constexpr int CNT = N / S::KSTEP + 1;  // kx values of a thread
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float2* areas = reinterpret_cast<float2*>(smem_raw);
     float2* t2 = reinterpret_cast<float2*>(smem_raw + S::tab_off);  // even-parity transpose twiddles
@@ -149,17 +160,49 @@ __global__ void __launch_bounds__(RowGroup<N>::NT, RowGroup<N>::MINB)
     const float2 wq = cconj(__ldg(tw + (q << shift_p)));  // W_P^-q
     const int s2 = tid % S::PAIRS, kx0 = S::first_kx(tid), r = kx0 & 1;
     float2* zp = areas + (2 * s2 + r) * S::AREA;
+    const size_t step = (size_t)S::KSTEP * O * i_pad;
     chain_wait();  // the half spectra are in place
+
+    // where tile t's rows of this thread start
+    auto place = [&](unsigned t, int& i0) {
+        const unsigned rest = t / rbs;
+        const int bz = (int)(rest / (unsigned)O), o = (int)(rest - (unsigned)bz * (unsigned)O);
+        i0 = (int)(t - rest * rbs) * S::ROWS + 2 * s2;
+        return bz * in_bstride + ((size_t)kx0 * O + o) * i_pad + (i0 < I ? i0 : 0);
+    };
+    // A, B at kx into bins kx and P - kx of Z = A + i B
+    auto put = [&](int kx, int i0, float4 v) {
+        if (i0 >= I) v.x = v.y = 0.f;
+        if (i0 + 1 >= I) v.z = v.w = 0.f;
+        if (kx == 0 || kx == N) v.y = v.w = 0.f;  // real DC and Nyquist
+        const int k = kx >> 1;
+        zp[k] = make_float2(v.x - v.w, v.y + v.z);
+        if (kx > 0 && kx < N) zp[r ? N - 1 - k : N - k] = make_float2(v.x + v.w, v.z - v.y);
+    };
+    float4 next[AHEAD ? CNT : 1];
+    auto fetch = [&](unsigned t) {
+        // every register is set on every path, so that none lives through the transform
+        const bool live = t < ntiles;
+        int i0;
+        const float2* src = in0 + place(live ? t : 0, i0);
+#pragma unroll
+        for (int i = 0; i < CNT; ++i)
+            next[AHEAD ? i : 0] = live && kx0 + i * S::KSTEP <= N ? load_here4_cg(src + i * step)
+                                                                : make_float4(0.f, 0.f, 0.f, 0.f);
+    };
+    if (AHEAD) fetch(blockIdx.x);
 
     for (unsigned t = blockIdx.x; t < ntiles; t += gridDim.x) {
         const unsigned rest = t / rbs;
         const int ib = (int)(t - rest * rbs) * S::ROWS;
         const int bz = (int)(rest / (unsigned)O), o = (int)(rest - (unsigned)bz * (unsigned)O);
-        {
-            const int i0 = ib + 2 * s2;
-            const bool ha = i0 < I, hb = i0 + 1 < I;
-            const size_t step = (size_t)S::KSTEP * O * i_pad;
-            size_t at = bz * in_bstride + ((size_t)kx0 * O + o) * i_pad + (ha ? i0 : 0);
+        int i0;
+        size_t at = place(t, i0);
+        if constexpr (AHEAD) {
+#pragma unroll
+            for (int i = 0; i < CNT; ++i)
+                if (kx0 + i * S::KSTEP <= N) put(kx0 + i * S::KSTEP, i0, next[i]);
+        } else {
 #pragma unroll 4
             for (int kx = kx0; kx <= N; kx += S::KSTEP, at += step) {
                 float4 v = __ldcg(reinterpret_cast<const float4*>(in0 + at));
@@ -167,12 +210,7 @@ __global__ void __launch_bounds__(RowGroup<N>::NT, RowGroup<N>::MINB)
                     const float4 w = __ldcg(reinterpret_cast<const float4*>(in1 + at));
                     v = make_float4(v.x + w.x, v.y + w.y, v.z + w.z, v.w + w.w);
                 }
-                if (!ha) v.x = v.y = 0.f;
-                if (!hb) v.z = v.w = 0.f;
-                if (kx == 0 || kx == N) v.y = v.w = 0.f;  // real DC and Nyquist
-                const int k = kx >> 1;
-                zp[k] = make_float2(v.x - v.w, v.y + v.z);  // A + i B
-                if (kx > 0 && kx < N) zp[r ? N - 1 - k : N - k] = make_float2(v.x + v.w, v.z - v.y);  // at P - kx
+                put(kx, i0, v);
             }
         }
         __syncthreads();
@@ -190,17 +228,18 @@ __global__ void __launch_bounds__(RowGroup<N>::NT, RowGroup<N>::MINB)
                 for (int e = 0; e < G::V; ++e) area[group_bin<N>(q, e)] = u[e];
             }
         }
+        if (AHEAD) fetch(t + gridDim.x);
         __syncthreads();
         // a warp stores 32 values of both rows of one pair at a time
         const int chunks = (l_out + 31) >> 5;
         for (int w = warp; w < S::PAIRS * chunks; w += S::WARPS) {
             const int sp = w / chunks, x = (w - sp * chunks) * 32 + lane;
-            const int i0 = ib + 2 * sp;
-            if (i0 < I && x < l_out) {
+            const int j0 = ib + 2 * sp;
+            if (j0 < I && x < l_out) {
                 const float2 z = cadd(areas[2 * sp * S::AREA + x], areas[(2 * sp + 1) * S::AREA + x]);
-                float* oa = out + bz * out_bstride + ((size_t)o * I + i0) * out_stride + x;
+                float* oa = out + bz * out_bstride + ((size_t)o * I + j0) * out_stride + x;
                 oa[0] = z.x;
-                if (i0 + 1 < I) oa[out_stride] = z.y;
+                if (j0 + 1 < I) oa[out_stride] = z.y;
             }
         }
         __syncthreads();  // the areas are rewritten by the next tile
@@ -208,8 +247,9 @@ __global__ void __launch_bounds__(RowGroup<N>::NT, RowGroup<N>::MINB)
 }
 
 // The y passes of the equal-dimension plans.  384 x 320 x 64 adjoint: forward
-// rows 599 -> 463 us (2.1 GB: 0.31 ms at the copy rate), inverse 95 -> 84 us
-// against block transforms.
+// rows 599 -> 428 us (2.1 GB: 0.31 ms at the copy rate; 463 us without the
+// next tile's loads in flight during the writes), inverse 95 -> 84 us, against
+// block transforms.
 //
 // Complex rows, l_in <= N values zero-padded to 2N points: row k of `in` to
 // row k of `out`, written as (Z(2k), Z(2k + 1)) pairs of 16 bytes.  A tile is
@@ -230,22 +270,25 @@ __global__ void __launch_bounds__(RowGroup<N>::NT, RowGroup<N>::MINB)
     build_group_tw<N>(tab + N, 1, tw, shift_p, tid, S::NT);
     __syncthreads();
     float2* area = areas + (2 * s + p) * S::AREA;
+    float2 u[G::V];
+    auto load = [&](unsigned t) {
+        const long row = (long)t * S::PAIRS + s;
+        const bool ok = row < rows;
+        const float2* src = in + (size_t)(ok ? row : 0) * in_stride;
+#pragma unroll
+        for (int n2 = 0; n2 < G::V; ++n2) {
+            const int x = q + G::L * n2;
+            u[n2] = ok && x < l_in ? load_here(src + x) : make_float2(0.f, 0.f);
+        }
+    };
+    load(blockIdx.x);
     for (unsigned t = blockIdx.x; t < ntiles; t += gridDim.x) {
         const long row0 = (long)t * S::PAIRS;
-        {
-            const bool ok = row0 + s < rows;
-            const float2* src = in + (size_t)(ok ? row0 + s : 0) * in_stride;
-            float2 u[G::V];
+        if (p) fold_regs<N>(u);
+        group_fft<N, false>(u, area, tab + p * N, q);
 #pragma unroll
-            for (int n2 = 0; n2 < G::V; ++n2) {
-                const int x = q + G::L * n2;
-                u[n2] = ok && x < l_in ? __ldg(src + x) : make_float2(0.f, 0.f);
-            }
-            if (p) fold_regs<N>(u);
-            group_fft<N, false>(u, area, tab + p * N, q);
-#pragma unroll
-            for (int e = 0; e < G::V; ++e) area[group_bin<N>(q, e)] = u[e];
-        }
+        for (int e = 0; e < G::V; ++e) area[group_bin<N>(q, e)] = u[e];
+        if (t + gridDim.x < ntiles) load(t + gridDim.x);  // in flight while this tile is written
         __syncthreads();
         for (int e = tid; e < S::PAIRS * N; e += S::NT) {
             const int sr = e / N, k = e % N;
@@ -274,23 +317,26 @@ __global__ void __launch_bounds__(RowGroup<N>::NT, RowGroup<N>::MINB)
     __syncthreads();
     float2* area = areas + (2 * s + p) * S::AREA;
     const float2 wq = cconj(__ldg(tw + (q << shift_p)));  // W_P^-q
+    float2 u[G::V];
+    auto load = [&](unsigned t) {
+        const long row = (long)t * S::PAIRS + s;
+        const bool ok = row < rows;
+        const float2* src = in + (size_t)(ok ? row : 0) * in_stride + p;
+#pragma unroll
+        for (int n2 = 0; n2 < G::V; ++n2) u[n2] = ok ? load_here(src + 2 * (q + G::L * n2)) : make_float2(0.f, 0.f);
+    };
+    load(blockIdx.x);
     for (unsigned t = blockIdx.x; t < ntiles; t += gridDim.x) {
         const long row0 = (long)t * S::PAIRS;
-        {
-            const bool ok = row0 + s < rows;
-            const float2* src = in + (size_t)(ok ? row0 + s : 0) * in_stride + p;
-            float2 u[G::V];
+        group_fft<N, true>(u, area, t2, q);
+        if (p) {
 #pragma unroll
-            for (int n2 = 0; n2 < G::V; ++n2) u[n2] = ok ? __ldg(src + 2 * (q + G::L * n2)) : make_float2(0.f, 0.f);
-            group_fft<N, true>(u, area, t2, q);
-            if (p) {
+            for (int e = 0; e < G::V; ++e) area[group_bin<N>(q, e)] = unfold_reg<N>(u[e], wq, e);
+        } else {
 #pragma unroll
-                for (int e = 0; e < G::V; ++e) area[group_bin<N>(q, e)] = unfold_reg<N>(u[e], wq, e);
-            } else {
-#pragma unroll
-                for (int e = 0; e < G::V; ++e) area[group_bin<N>(q, e)] = u[e];
-            }
+            for (int e = 0; e < G::V; ++e) area[group_bin<N>(q, e)] = u[e];
         }
+        if (t + gridDim.x < ntiles) load(t + gridDim.x);  // in flight while this tile is written
         __syncthreads();
         const int chunks = (l_out + 31) >> 5;
         for (int w = warp; w < S::PAIRS * chunks; w += S::WARPS) {
@@ -348,11 +394,11 @@ cudaError_t r2c_launch(const float* in, size_t in_ostride, size_t in_istride, in
     return cudaGetLastError();
 }
 
-template <int N>
+template <int N, bool AHEAD>
 cudaError_t c2r_launch(const void* in0, const void* in1, int I, int O, int i_pad, float* out, size_t out_stride,
                        int l_out, const void* tw, int log_t, cudaStream_t s, Batch b) {
     using S = RowGroup<N>;
-    constexpr auto k = row_c2r_group_kernel<N>;
+    constexpr auto k = row_c2r_group_kernel<N, AHEAD>;
     constexpr size_t smem = S::tab_off + N * sizeof(float2);
     cudaError_t e = ensure_smem_limit<k>();
     if (e != cudaSuccess) return e;
@@ -366,6 +412,15 @@ cudaError_t c2r_launch(const void* in0, const void* in1, int I, int O, int i_pad
     return launch_chained(k, dim3((unsigned)std::min(ntiles, fill)), S::NT, smem, s, (const float2*)in0,
                           (const float2*)in1, I, O, i_pad, out, out_stride, l_out, (const float2*)tw, shift_p, b.in,
                           b.out, (unsigned)ntiles, rbs);
+}
+
+template <int N>
+cudaError_t c2r_either(const void* in0, const void* in1, int I, int O, int i_pad, float* out, size_t out_stride,
+                       int l_out, const void* tw, int log_t, cudaStream_t s, Batch b) {
+    if constexpr (N >= 512) {
+        if (!in1) return c2r_launch<N, true>(in0, in1, I, O, i_pad, out, out_stride, l_out, tw, log_t, s, b);
+    }
+    return c2r_launch<N, false>(in0, in1, I, O, i_pad, out, out_stride, l_out, tw, log_t, s, b);
 }
 
 template <int N>
@@ -429,11 +484,11 @@ cudaError_t launch_row_c2r_group(int log_p, const void* in0, const void* in1, in
         !aligned16(in1))
         return cudaErrorNotSupported;
     switch (log_p) {
-        case 7: return c2r_launch<64>(in0, in1, I, O, i_pad, out, out_stride, l_out, tw, log_t, s, b);
-        case 8: return c2r_launch<128>(in0, in1, I, O, i_pad, out, out_stride, l_out, tw, log_t, s, b);
-        case 9: return c2r_launch<256>(in0, in1, I, O, i_pad, out, out_stride, l_out, tw, log_t, s, b);
-        case 10: return c2r_launch<512>(in0, in1, I, O, i_pad, out, out_stride, l_out, tw, log_t, s, b);
-        default: return c2r_launch<1024>(in0, in1, I, O, i_pad, out, out_stride, l_out, tw, log_t, s, b);
+        case 7: return c2r_either<64>(in0, in1, I, O, i_pad, out, out_stride, l_out, tw, log_t, s, b);
+        case 8: return c2r_either<128>(in0, in1, I, O, i_pad, out, out_stride, l_out, tw, log_t, s, b);
+        case 9: return c2r_either<256>(in0, in1, I, O, i_pad, out, out_stride, l_out, tw, log_t, s, b);
+        case 10: return c2r_either<512>(in0, in1, I, O, i_pad, out, out_stride, l_out, tw, log_t, s, b);
+        default: return c2r_either<1024>(in0, in1, I, O, i_pad, out, out_stride, l_out, tw, log_t, s, b);
     }
 }
 

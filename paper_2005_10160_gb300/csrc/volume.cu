@@ -200,16 +200,20 @@ __global__ void __launch_bounds__(kYwThreads, 2)
     float2* tr = areas + warp * kYwArea;
     const float2* za = areas + 2 * sq * kYwArea;  // Z(2k) of this row
     const float2* zb = za + kYwArea;              // Z(2k + 1)
-    for (long g = blockIdx.x; g * kYwRows < rows; g += gridDim.x) {
-        const long row = g * kYwRows + sq;
+    float2 u[32];
+    auto load = [&](long row) {
         const bool ok = row < rows;
         const float2* src = in + (size_t)(ok ? row : 0) * in_stride;
-        float2 u[32];
 #pragma unroll
         for (int n1 = 0; n1 < 32; ++n1) {
             const int y = 32 * n1 + lane;
-            u[n1] = (ok && y < l_in) ? src[y] : make_float2(0.f, 0.f);
+            u[n1] = (ok && y < l_in) ? load_here(src + y) : make_float2(0.f, 0.f);
         }
+    };
+    load((long)blockIdx.x * kYwRows + sq);
+    for (long g = blockIdx.x; g * kYwRows < rows; g += gridDim.x) {
+        const long row = g * kYwRows + sq;
+        const bool ok = row < rows;
         if (p) {
 #pragma unroll
             for (int n1 = 0; n1 < 32; ++n1) u[n1] = cmul(u[n1], t1[32 * n1 + lane]);
@@ -217,6 +221,7 @@ __global__ void __launch_bounds__(kYwThreads, 2)
         warp_fft1024<false>(u, tr, t2, lane);  // u[j] = Z(2 (lane + 32 bitrev5(j)) + p)
 #pragma unroll
         for (int j = 0; j < 32; ++j) tr[lane + 32 * bitrev5(j)] = u[j];
+        load((g + gridDim.x) * kYwRows + sq);  // the next row, in flight while this one is written
         pair_sync(1 + sq);
         if (ok) {
             float4* dst = reinterpret_cast<float4*>(out + (size_t)row * out_stride);
@@ -246,14 +251,17 @@ __global__ void __launch_bounds__(kYwThreads, 2)
     const int kxg = (kx_count + kYwRows - 1) / kYwRows;
     const int ybs = (ny + 7) >> 3;
     const unsigned groups = (unsigned)kxg * (unsigned)R;  // at most 257 x 4608
+    float2 u[32];
+    auto load = [&](unsigned g) {
+        const int r = (int)(g / (unsigned)kxg), kx = (int)(g - (unsigned)r * (unsigned)kxg) * kYwRows + sq;
+        const bool ok = g < groups && kx < kx_count;
+        const float2* src = in + (ok ? ((size_t)kx * R + r) * 2048 : 0) + p;
+#pragma unroll
+        for (int n1 = 0; n1 < 32; ++n1) u[n1] = ok ? load_here(src + 2 * (32 * n1 + lane)) : make_float2(0.f, 0.f);
+    };
+    load(blockIdx.x);
     for (unsigned g = blockIdx.x; g < groups; g += gridDim.x) {
         const int r = (int)(g / (unsigned)kxg), kx0 = (int)(g - (unsigned)r * (unsigned)kxg) * kYwRows;
-        const int kx = kx0 + sq;
-        const bool ok = kx < kx_count;
-        const float2* src = in + ((size_t)(ok ? kx : 0) * R + r) * 2048 + p;
-        float2 u[32];
-#pragma unroll
-        for (int n1 = 0; n1 < 32; ++n1) u[n1] = ok ? src[2 * (32 * n1 + lane)] : make_float2(0.f, 0.f);
         warp_fft1024<true>(u, tr, t2, lane);  // u[j] = E or O at m = lane + 32 bitrev5(j)
         if (p) {
 #pragma unroll
@@ -261,6 +269,7 @@ __global__ void __launch_bounds__(kYwThreads, 2)
         }
 #pragma unroll
         for (int j = 0; j < 32; ++j) tr[lane + 32 * bitrev5(j)] = u[j];
+        load(g + gridDim.x);  // the next group's rows, in flight while this one is written
         __syncthreads();  // E and W^-m O of all four rows are in place
         {
             // thread tid writes slot tid % 8 of row kx0 + (tid / 8) % 4 in the
