@@ -213,7 +213,7 @@ int make_spectra(grav_plan* p) {
         } else {
             const Geometry g{p->nx, p->ny, p->nz, p->dx, p->dy, p->dz, p->h};
             SpecBuild b{p->nx, p->ny, p->nz, ny2, p->ncomp, p->kx_count, p->jp, p->log_px, p->log_py, 0, p->oddv_mask};
-            GenOut o = gen_out(p->fp64 ? GenOut::kQuadrant : GenOut::kQuadrantPairs);
+            GenOut o = gen_out(p->fp64 ? GenOut::kQuadrant : GenOut::kQuadrantPairs, !p->fp64);
             double factor[kMaxPlanComp];
             // FP32 pairs: kernels in units of upsilon (times the largest cell
             // edge for first derivatives), which are of order 1 at most
@@ -588,7 +588,7 @@ int grav_kernel_values(int nx, int ny, int nz, double dx, double dy, double dz, 
         return GRAV_EINVAL;
     }
     Geometry g{nx, ny, nz, dx, dy, dz, h};
-    cudaError_t e = launch_kernel_gen(g, gen_out(GenOut::kOffsets), components & kCompBits, 0, nz, K_dev, (cudaStream_t)stream);
+    cudaError_t e = launch_kernel_gen(g, gen_out(GenOut::kOffsets, false), components & kCompBits, 0, nz, K_dev, (cudaStream_t)stream);
     if (e != cudaSuccess) return cuda_fail(e, "kernel generation launch");
     return GRAV_OK;
 }

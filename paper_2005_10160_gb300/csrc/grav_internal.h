@@ -199,11 +199,12 @@ struct GenOut {
         kQuadrantPairs,  // the same as unevaluated FP32 pairs (float2)
     };
     Mode mode;
+    bool tables;             // the faster corner terms, for values that end up in FP32 spectra
     int px, py;              // kHalfRows
     double factor[kMaxComp];  // value = factor[component] times the corner sum (upsilon for SI units)
 };
 // Output of the given mode in SI units.
-GenOut gen_out(GenOut::Mode mode, int px = 0, int py = 0);
+GenOut gen_out(GenOut::Mode mode, bool tables, int px = 0, int py = 0);
 // Layers n0 .. n1 (nzc = n1 - n0), one slot per selected component.
 cudaError_t launch_kernel_gen(const Geometry& g, const GenOut& o, unsigned comps, int n0, int n1, void* out,
                               cudaStream_t s);

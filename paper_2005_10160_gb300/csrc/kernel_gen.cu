@@ -52,17 +52,37 @@ __device__ __forceinline__ Dist distance(double a, double b) {
 // NC: components kept per corner, 7 (gz ... gzz) or 9 (with gx, gy); plans
 // without gx, gy use 7 so that the kernel keeps fewer registers.  rxy, rxz,
 // ryz: distances in the coordinate planes.
-template <int NC>
-__device__ __forceinline__ void corner_terms(double x, double y, double z, double r, Dist rxy, Dist rxz, Dist ryz,
-                                             unsigned comps, const CornerTables& t, double (&F)[NC]) {
+//
+// TABLES (plans that store FP32 spectra): corner_terms.cuh and the shared
+// distances, whose rounding is up to 1.23 times that of the other form for
+// some components (0.87 to 0.95 for gz), far below FP32's.  Otherwise (FP64
+// plans, kernel values) CUDA's asinh and atan, 2.3 times the FP64
+// instructions.
+template <int NC, bool TABLES>
+__device__ __forceinline__ void corner_terms(double x, double y, double z, const Dist* rxy, const Dist* rxz,
+                                             const Dist* ryz, unsigned comps, const CornerTables& t,
+                                             double (&F)[NC]) {
+    const bool want_ay = comps & (GRAV_GZ | GRAV_GXZ | GRAV_GX), want_ax = comps & (GRAV_GZ | GRAV_GYZ | GRAV_GY),
+               want_az = comps & (GRAV_GXY | GRAV_GX | GRAV_GY), want_tz = comps & (GRAV_GZ | GRAV_GZZ),
+               want_tx = comps & (GRAV_GXX | GRAV_GX), want_ty = comps & (GRAV_GYY | GRAV_GY);
+    const double x2 = x * x, y2 = y * y, z2 = z * z, r = sqrt(x2 + y2 + z2);
     double ay = 0.0, ax = 0.0, az = 0.0, tz = 0.0, tx = 0.0, ty = 0.0;
-    const double xa = fabs(x), ya = fabs(y), za = fabs(z);
-    if (comps & (GRAV_GZ | GRAV_GXZ | GRAV_GX)) ay = asinh_ratio(y, rxz.inv, r + rxz.d, t);
-    if (comps & (GRAV_GZ | GRAV_GYZ | GRAV_GY)) ax = asinh_ratio(x, ryz.inv, r + ryz.d, t);
-    if (comps & (GRAV_GXY | GRAV_GX | GRAV_GY)) az = asinh_ratio(z, rxy.inv, r + rxy.d, t);
-    if (comps & (GRAV_GZ | GRAV_GZZ)) tz = copysign(atan_ratio(xa * ya, za * r, t), x * y * z);
-    if (comps & (GRAV_GXX | GRAV_GX)) tx = copysign(atan_ratio(ya * za, xa * r, t), x * y * z);
-    if (comps & (GRAV_GYY | GRAV_GY)) ty = copysign(atan_ratio(xa * za, ya * r, t), x * y * z);
+    if constexpr (TABLES) {
+        const double xa = fabs(x), ya = fabs(y), za = fabs(z);
+        if (want_ay) ay = asinh_ratio(y, rxz->inv, r + rxz->d, t);
+        if (want_ax) ax = asinh_ratio(x, ryz->inv, r + ryz->d, t);
+        if (want_az) az = asinh_ratio(z, rxy->inv, r + rxy->d, t);
+        if (want_tz) tz = copysign(atan_ratio(xa * ya, za * r, t), x * y * z);
+        if (want_tx) tx = copysign(atan_ratio(ya * za, xa * r, t), x * y * z);
+        if (want_ty) ty = copysign(atan_ratio(xa * za, ya * r, t), x * y * z);
+    } else {
+        if (want_ay) ay = asinh(y / sqrt(x2 + z2));
+        if (want_ax) ax = asinh(x / sqrt(y2 + z2));
+        if (want_az) az = asinh(z / sqrt(x2 + y2));
+        if (want_tz) tz = atan(x * y / (z * r));
+        if (want_tx) tx = atan(y * z / (x * r));
+        if (want_ty) ty = atan(x * z / (y * r));
+    }
     F[0] = -(x * ay + y * ax - z * tz);
     F[1] = tx;
     F[2] = -az;
@@ -94,8 +114,8 @@ __device__ __forceinline__ float2 split_pair(double v) {
 // above in shared memory, and every thread forms its offsets' kernel values
 // from four differences.  blockIdx.z takes a run of `per` layers.
 //
-// Bound by FP64 issue.  512 x 512 x 64, six components: 14.7 ms with the
-// library's asinh and atan, tiles of 32 x 8 and one run of layers.
+// Bound by FP64 issue.  1024 x 1024 x 100, six components: 65 ms with the
+// tables, 92 ms with the library's asinh and atan and tiles of 32 x 8.
 constexpr int kGenTX = 32, kGenTY = 16, kGenThreads = 256;
 constexpr int kGenCX = kGenTX + 1, kGenCY = kGenTY + 1, kGenCor = kGenCX * kGenCY;
 constexpr size_t gen_smem(int nc) {
@@ -103,7 +123,7 @@ constexpr size_t gen_smem(int nc) {
            (size_t)(kGenCor + kGenCX + kGenCY) * sizeof(Dist);
 }
 
-template <int NC>
+template <int NC, bool TABLES>
 __global__ void __launch_bounds__(kGenThreads)
     kernel_gen(Geometry g, GenOut o, unsigned comps, int n0, int n1, int per, void* __restrict__ out) {
     constexpr int CX = kGenCX, NT = kGenThreads;
@@ -122,21 +142,22 @@ __global__ void __launch_bounds__(kGenThreads)
     // corner (cx, cy) sits at x = (1/2 - u0 - cx) dx, y = (1/2 - v0 - cy) dy (station at the origin)
     auto cx_of = [&](int cx) { return (0.5 - (u0 + cx)) * g.dx; };
     auto cy_of = [&](int cy) { return (0.5 - (v0 + cy)) * g.dy; };
-    for (int e = tid; e < CornerTables::LOGS; e += NT) corner_table_entry(tab, e);
-    for (int e = tid; e < kGenCor; e += NT) {
-        rxy[e] = distance(cx_of(e % CX), cy_of(e / CX));
+    if constexpr (TABLES) {
+        for (int e = tid; e < CornerTables::LOGS; e += NT) corner_table_entry(tab, e);
+        for (int e = tid; e < kGenCor; e += NT) rxy[e] = distance(cx_of(e % CX), cy_of(e / CX));
     }
     // corner terms of z-level z into F and, but for the first level, their change into D
     auto level = [&](double z, bool difference) {
-        if (tid < CX) rxz[tid] = distance(cx_of(tid), z);
-        else if (tid >= 64 && tid < 64 + kGenCY) ryz[tid - 64] = distance(cy_of(tid - 64), z);
+        if constexpr (TABLES) {
+            if (tid < CX) rxz[tid] = distance(cx_of(tid), z);
+            else if (tid >= 64 && tid < 64 + kGenCY) ryz[tid - 64] = distance(cy_of(tid - 64), z);
+        }
         __syncthreads();  // distances in place; D and the tables free or in place
         for (int e = tid; e < kGenCor; e += NT) {
             const int cy = e / CX, cx = e - cy * CX;
             if (u0 + cx > g.nx || v0 + cy > g.ny) continue;
             double t[NC];
-            const double x = cx_of(cx), y = cy_of(cy);
-            corner_terms<NC>(x, y, z, sqrt(x * x + y * y + z * z), rxy[e], rxz[cx], ryz[cy], comps, tab, t);
+            corner_terms<NC, TABLES>(cx_of(cx), cy_of(cy), z, rxy + e, rxz + cx, ryz + cy, comps, tab, t);
 #pragma unroll
             for (int c = 0; c < NC; ++c) {
                 if (!(comps & (1u << c))) continue;
@@ -195,9 +216,9 @@ __global__ void __launch_bounds__(kGenThreads)
     }
 }
 
-template <int NC>
+template <int NC, bool TABLES>
 cudaError_t gen_launch(const Geometry& g, const GenOut& o, unsigned comps, int n0, int n1, void* out, cudaStream_t s) {
-    constexpr auto k = kernel_gen<NC>;
+    constexpr auto k = kernel_gen<NC, TABLES>;
     cudaError_t e = ensure_smem_limit<k>();
     if (e != cudaSuccess) return e;
     dim3 grid((g.nx + kGenTX - 1) / kGenTX, (g.ny + kGenTY - 1) / kGenTY);
@@ -216,13 +237,16 @@ cudaError_t gen_launch(const Geometry& g, const GenOut& o, unsigned comps, int n
 cudaError_t launch_kernel_gen(const Geometry& g, const GenOut& o, unsigned comps, int n0, int n1, void* out,
                               cudaStream_t s) {
     comps &= kCompBits;
-    return comps & (GRAV_GX | GRAV_GY) ? gen_launch<9>(g, o, comps, n0, n1, out, s)
-                                       : gen_launch<7>(g, o, comps, n0, n1, out, s);
+    const bool nine = comps & (GRAV_GX | GRAV_GY);
+    if (o.tables)
+        return nine ? gen_launch<9, true>(g, o, comps, n0, n1, out, s) : gen_launch<7, true>(g, o, comps, n0, n1, out, s);
+    return nine ? gen_launch<9, false>(g, o, comps, n0, n1, out, s) : gen_launch<7, false>(g, o, comps, n0, n1, out, s);
 }
 
-GenOut gen_out(GenOut::Mode mode, int px, int py) {
+GenOut gen_out(GenOut::Mode mode, bool tables, int px, int py) {
     GenOut o{};
     o.mode = mode;
+    o.tables = tables;
     o.px = px;
     o.py = py;
     for (double& f : o.factor) f = kUpsilon;

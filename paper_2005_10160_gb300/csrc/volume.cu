@@ -1065,7 +1065,7 @@ int make_spectra3(grav_plan* p) {
                         rc = cuda_fail(ce, "cudaMemsetAsync(kernel staging)");
                         break;
                     }
-                    if ((ce = launch_kernel_gen(g, gen_out(GenOut::kHalfRows, p->px, p->py), 1u << c, j0, j1, E, s)) != cudaSuccess) {
+                    if ((ce = launch_kernel_gen(g, gen_out(GenOut::kHalfRows, !p->fp64, p->px, p->py), 1u << c, j0, j1, E, s)) != cudaSuccess) {
                         rc = cuda_fail(ce, "kernel generation launch");
                         break;
                     }
