@@ -3,7 +3,7 @@
 // has: register transforms by groups of lanes (group_fft.cuh), one for the
 // even and one for the odd bins of each packed row pair a + i b.
 //
-// A tile is 8 row pairs (4 for P = 2048) of one layer; warps of even index
+// A tile is 8 row pairs of one layer (4 for P = 2048, but for the forward rows); warps of even index
 // run the even bins, warps of odd index the odd ones, so the fold of the odd
 // bins is a warp-uniform branch.  Tiles are walked by a grid that fills the
 // machine once, so the twiddle tables are built once per CTA, and the next
@@ -13,14 +13,17 @@
 // hits L1).
 //
 // The areas of the transforms start 1 complex value apart modulo 16 (2 for
-// P = 2048) and the pairs of a warp are chosen so that the 16 lanes of each
+// tiles of 4 pairs) and the pairs of a warp are chosen so that the 16 lanes of each
 // shared-memory phase fall in different banks, in the transposes as well as
 // in the passes across pairs.
 //
 // Against the block FFTs through shared memory that they replaced: 256-value
 // rows of 32 layers 11.7 -> 8.9 us, 16 requests of 128-value rows 38.9 -> 24.5,
 // 301-value rows of 45 layers 35.7 -> 18.2, their inverse 52.4 -> 30.9 (from
-// one summed input instead of two).  Issue slots are half busy; the rest waits
+// one summed input instead of two).  1024-value rows of 100 layers: 310 us, 4.1
+// TB/s (a kernel of one warp a transform, its rows staged by bulk copies, 313;
+// tiles of 4 pairs 317; the inverse rows of six planes are the other way round,
+// 48 us in tiles of 4 pairs, 51 of 8).  Issue slots are half busy; the rest waits
 // on the shared-memory transposes and the two barriers a tile.
 #include <climits>
 #include <algorithm>
@@ -33,13 +36,13 @@ namespace grav {
 
 namespace {
 
-template <int N> struct RowGroup {
+template <int N, int PAIRS_ = (N >= 1024 ? 4 : 8)> struct RowGroup {
     using G = GroupFft<N>;
-    static constexpr int PAIRS = N >= 1024 ? 4 : 8;               // row pairs of a tile
+    static constexpr int PAIRS = PAIRS_;                          // row pairs of a tile
     static constexpr int ROWS = 2 * PAIRS;
     static constexpr int WARPS = 2 * PAIRS / G::GPW;
     static constexpr int NT = 32 * WARPS;
-    static constexpr int AREA = N >= 1024 ? G::TR + 2 : (G::TR + 15) / 16 * 16 + 1;
+    static constexpr int AREA = PAIRS == 4 ? G::TR + 2 : (G::TR + 15) / 16 * 16 + 1;
     static constexpr int KW = 32 / PAIRS;                         // kx values a warp covers
     static constexpr int KSTEP = NT / PAIRS;                      // kx values the CTA covers
     static constexpr size_t tab_off = (size_t)2 * PAIRS * AREA * sizeof(float2);
@@ -61,13 +64,16 @@ template <int N> struct RowGroup {
     }
 };
 
-// Real rows -> half spectra, written transposed (see launch_row_r2c).
+// Real rows -> half spectra, written transposed (see launch_row_r2c), in tiles
+// of 16 rows at every size: 128-byte runs.
+template <int N> using ForwardRows = RowGroup<N, 8>;
+
 template <int N>
-__global__ void __launch_bounds__(RowGroup<N>::NT, RowGroup<N>::MINB)
+__global__ void __launch_bounds__(ForwardRows<N>::NT, ForwardRows<N>::MINB)
     row_r2c_group_kernel(const float* __restrict__ in, size_t in_ostride, size_t in_istride, int l_in, int I, int O,
                          float2* __restrict__ out, int i_pad, const float2* __restrict__ tw, int shift_p,
                          size_t in_bstride, size_t out_bstride, unsigned ntiles, unsigned rbs) {
-    using S = RowGroup<N>;
+    using S = ForwardRows<N>;
     using G = GroupFft<N>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float2* areas = reinterpret_cast<float2*>(smem_raw);                // area of (pair s, parity p): 2 s + p
@@ -376,7 +382,7 @@ int resident_ctas(int nt, size_t smem) {
 template <int N>
 cudaError_t r2c_launch(const float* in, size_t in_ostride, size_t in_istride, int l_in, int I, int O, void* out,
                        int i_pad, const void* tw, int log_t, cudaStream_t s, Batch b) {
-    using S = RowGroup<N>;
+    using S = ForwardRows<N>;
     constexpr auto k = row_r2c_group_kernel<N>;
     constexpr size_t smem = S::tab_off + 2 * N * sizeof(float2);
     cudaError_t e = ensure_smem_limit<k>();

@@ -89,7 +89,7 @@ int forward_static(grav_plan* p, const void* rho, void* out, unsigned char* scra
     void* X = scratch;
     void* Y = scratch + x_bytes;
     cudaError_t e = launch_row_r2c<R>(p->log_px, (const R*)rho, (size_t)p->ny * p->nx, (size_t)p->nx, p->nx, p->ny,
-                                      p->nz, X, p->ny_pad, p->tw, p->log_t, s, Batch(), p->err_flag);
+                                      p->nz, X, p->ny_pad, p->tw, p->log_t, s, Batch());
     if (e != cudaSuccess) return cuda_fail(e, "static-scratch forward row transform");
     ColumnArgs a{p->ny, p->ny_pad, p->nz, p->ncomp, p->kx_count, p->jp, p->imag_mask, p->oddv_mask,
                  p->log_t - (p->log_py - 1), p->log_t - p->log_py};

@@ -1124,7 +1124,7 @@ int run_forward3d(grav_plan* p, const void* rho, void* out, cudaStream_t s) {
     cudaError_t e;
     // A: x
     e = launch_row_r2c<R>(p->log_px, (const R*)rho, (size_t)p->ny * p->nx, (size_t)p->nx, p->nx, p->ny, p->nz, A,
-                          p->ny_pad, p->tw, p->log_t, s, Batch(), p->err_flag);
+                          p->ny_pad, p->tw, p->log_t, s);
     if (e != cudaSuccess) return cuda_fail(e, "equal-dimension forward: row transforms");
     // B: y
     e = launch_vol_yfwd<C>(p->log_py, A, p->ny_pad, p->ny, B, p->py, (long)(kx * nz), p->tw, p->log_t, s);
@@ -1161,7 +1161,7 @@ int run_adjoint3d(grav_plan* p, const void* r, void* grad, cudaStream_t s) {
     void* B = p->ws_b;
     cudaError_t e;
     e = launch_row_r2c<R>(p->log_px, (const R*)r, (size_t)p->ny * p->nx, (size_t)p->nx, p->nx, p->ny, (int)(nc * nz),
-                          A, p->ny_pad, p->tw, p->log_t, s, Batch(), p->err_flag);
+                          A, p->ny_pad, p->tw, p->log_t, s);
     if (e != cudaSuccess) return cuda_fail(e, "equal-dimension adjoint: row transforms");
     e = launch_vol_yfwd<C>(p->log_py, A, p->ny_pad, p->ny, B, p->py, (long)(kx * nc * nz), p->tw, p->log_t, s);
     if (e != cudaSuccess) return cuda_fail(e, "equal-dimension adjoint: column transforms");
