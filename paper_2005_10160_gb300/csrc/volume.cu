@@ -862,12 +862,20 @@ cudaError_t launch_vol_yinv_tiled(int logn, const void* in, int R, int kx_count,
     }
 }
 
+// Whether rows of 2^logn values are transformed by the lane-group kernels.
+template <typename C>
+constexpr bool lane_group_rows(int logn) {
+    return std::is_same<C, float2>::value && logn >= 7 && logn <= 11;
+}
+
 template <typename C, bool INV>
 cudaError_t launch_vol_rows(int logn, const void* in, size_t in_stride, int l_in, void* out, size_t out_stride,
                             int l_out, long rows, const void* tw, int log_t, cudaStream_t s) {
     switch (logn) {
 #define CASE(L) \
-    case L: return rows_launch<C, L, INV>(in, in_stride, l_in, out, out_stride, l_out, rows, tw, log_t - L, s);
+    case L:                                                                                                         \
+        if constexpr (lane_group_rows<C>(L)) return cudaErrorInvalidValue;                                          \
+        else return rows_launch<C, L, INV>(in, in_stride, l_in, out, out_stride, l_out, rows, tw, log_t - L, s);
         GRAV_VOL_LOG_CASES(CASE)
 #undef CASE
         default: return cudaErrorInvalidValue;
@@ -892,8 +900,9 @@ cudaError_t launch_vol_yfwd(int logn, const void* in, size_t in_stride, int l_in
         }
     }
     if constexpr (std::is_same<C, float2>::value) {
-        const cudaError_t e = launch_rows_fwd_group(logn, in, in_stride, l_in, out, out_stride, rows, tw, log_t, s);
-        if (e != cudaErrorNotSupported) return e;
+        // every plan's rows and workspaces satisfy its conditions
+        if (lane_group_rows<C>(logn))
+            return launch_rows_fwd_group(logn, in, in_stride, l_in, out, out_stride, rows, tw, log_t, s);
     }
     return launch_vol_rows<C, false>(logn, in, in_stride, l_in, out, out_stride, (int)out_stride, rows, tw, log_t, s);
 }
@@ -904,8 +913,8 @@ template <typename C>
 cudaError_t launch_vol_yinv(int logn, const void* in, size_t in_stride, void* out, size_t out_stride, int l_out,
                             long rows, const void* tw, int log_t, cudaStream_t s) {
     if constexpr (std::is_same<C, float2>::value) {
-        const cudaError_t e = launch_rows_inv_group(logn, in, in_stride, out, out_stride, l_out, rows, tw, log_t, s);
-        if (e != cudaErrorNotSupported) return e;
+        if (lane_group_rows<C>(logn))
+            return launch_rows_inv_group(logn, in, in_stride, out, out_stride, l_out, rows, tw, log_t, s);
     }
     return launch_vol_rows<C, true>(logn, in, in_stride, 1 << logn, out, out_stride, l_out, rows, tw, log_t, s);
 }
