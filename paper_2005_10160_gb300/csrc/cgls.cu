@@ -22,8 +22,10 @@
 // (step_model 174 us at 512 x 512 x 64 for 0.34 GB).  A thread therefore keeps
 // an FP32 plan's sum as an unevaluated pair of floats: the product's rounding
 // error by fused multiply-add, the sum's by the two-sum of Knuth (TAOCP 2,
-// 4.2.2), both added to the low part; products are exact and the sum is good
-// to about 2^-45, more than the separately rounded FP32 products had before.
+// 4.2.2), both added to the low part; the sum is good to about 2^-45, more than
+// that of separately rounded FP32 products.  A pair has FP32's range: sums from
+// 2^100 on move to an FP64 number, and the rounding error of a square below
+// about 1e-32 is lost, as in an FP32 product.
 #include <algorithm>
 
 #include "grav_internal.h"
@@ -85,17 +87,22 @@ template <> struct Squares<double> {
 };
 template <> struct Squares<float> {
     float hi = 0.f, lo = 0.f;
+    double big = 0.0;
     __device__ __forceinline__ void add(float v) {
         const float p = __fmul_rn(v, v), pe = __fmaf_rn(v, v, -p);
         const float t = __fadd_rn(hi, p), z = __fsub_rn(t, hi);
         const float te = __fadd_rn(__fsub_rn(hi, __fsub_rn(t, z)), __fsub_rn(p, z));
         hi = t;
         lo = __fadd_rn(lo, __fadd_rn(pe, te));
+        // a finite square added to less than 2^100 stays finite
+        if (hi >= 0x1p100f) {
+            big += pair();
+            hi = lo = 0.f;
+        }
     }
-    __device__ __forceinline__ double get() const {
-        // past the FP32 range the corrections are not numbers; the sum is
-        return isfinite(lo) ? (double)hi + (double)lo : (double)hi;
-    }
+    // past the FP32 range (an infinite square) the corrections are not numbers; the sum is
+    __device__ __forceinline__ double pair() const { return isfinite(lo) ? (double)hi + (double)lo : (double)hi; }
+    __device__ __forceinline__ double get() const { return big + pair(); }
 };
 
 template <typename R, int VEC> struct alignas(sizeof(R) * VEC) Pack { R v[VEC]; };
