@@ -170,7 +170,10 @@ int grav_adjoint_batch_plans(int batch, grav_plan* const* plans, const void* r_d
  * conjugate gradients on the normal equations in x = W_m m from x = 0, one
  * forward and one adjoint per step.  All scalars stay on the device: nothing
  * waits for the host.  When (s, s) is exactly 0 the remaining steps change
- * nothing.
+ * nothing.  After the steps the first int of work_dev is 0; 1: a step with
+ * (s, s) > 0 had no length, (q, q) + lam (p, p) being exactly 0 (squares below
+ * the element type's range); 2: a step's length was past the element type's
+ * range.  After 1 or 2 the later models and objectives are not numbers.
  *   d_dev           device [ncomp][ny][nx] data
  *   w_dev           device [ncomp][ny][nx] data weights (1 / sigma)
  *   wm_dev          device [nz] depth weights of the layers

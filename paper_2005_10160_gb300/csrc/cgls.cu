@@ -107,10 +107,14 @@ template <> struct Squares<float> {
 
 template <typename R, int VEC> struct alignas(sizeof(R) * VEC) Pack { R v[VEC]; };
 
+// What the steps found, the first int of the workspace.
+enum { kStepsDone = 0, kNoStepLength = 1, kStepLengthRange = 2 };
+
 // (s, s) before the step, (p, p), (q, q)
 struct Scalars {
     const Dot *gamma, *pp, *qq;
     double lam;
+    int* status;
 };
 // alpha, the same value in every thread.  A vanished gradient ends the
 // recurrence: nothing moves any more.
@@ -150,11 +154,17 @@ __global__ void __launch_bounds__(kVecThreads) cgls_weigh(const R* __restrict__ 
     put_dot(qq, s.get());
 }
 
-// r -= alpha q, wr = w r, (r, r)
+// r -= alpha q, wr = w r, (r, r); records a step without a length (a gradient,
+// but (q, q) + lam (p, p) = 0) or with one past R's range
 template <typename R>
 __global__ void __launch_bounds__(kVecThreads) cgls_step_data(Scalars k, const R* __restrict__ w, const R* __restrict__ q, R* __restrict__ r,
                                                               R* __restrict__ wr, size_t n, Dot* rr) {
-    const R alpha = (R)step_length(k);
+    const double step = step_length(k);
+    const R alpha = (R)step;
+    if (blockIdx.x == 0 && threadIdx.x == 0 && *k.status == kStepsDone) {
+        if (k.gamma->value != 0.0 && k.qq->value + k.lam * k.pp->value == 0.0) *k.status = kNoStepLength;
+        else if (!isinf(step) && isinf(alpha)) *k.status = kStepLengthRange;
+    }
     Squares<R> s;
     for (size_t i = (size_t)blockIdx.x * kVecThreads + threadIdx.x; i < n; i += (size_t)gridDim.x * kVecThreads) {
         const R v = r[i] - alpha * q[i];
@@ -267,13 +277,15 @@ __global__ void __launch_bounds__(kVecThreads) cgls_objectives(const Dot* dots, 
 
 size_t pad256(size_t v) { return (v + 255) / 256 * 256; }
 
-// The caller's workspace: data vectors r, q, wr; model vectors p, t, g, x; then
-// the dot products: (p, p), (q, q) and, per step, (r, r), (x, x), (s, s).
+// The caller's workspace: the status; data vectors r, q, wr; model vectors p, t,
+// g, x; then the dot products: (p, p), (q, q) and, per step, (r, r), (x, x),
+// (s, s).
 struct Work {
+    static constexpr size_t kHead = 256;  // the status
     size_t nd, plane, data, model;
     int nz, iters;
     size_t dots() const { return 2 + 3 * ((size_t)iters + 1); }
-    size_t bytes() const { return 3 * data + 4 * model + dots() * sizeof(Dot); }
+    size_t bytes() const { return kHead + 3 * data + 4 * model + dots() * sizeof(Dot); }
 };
 Work work_of(const grav_plan* p, int iters) {
     Work w{};
@@ -289,13 +301,15 @@ Work work_of(const grav_plan* p, int iters) {
 
 template <typename R> struct Loop {
     Work k;
+    int* status;
     R *r, *q, *wr, *p, *t, *g, *x;
     Dot *pp, *qq, *step;
     unsigned gd;      // blocks of the data-size kernels
     dim3 gm;          // blocks of the model-size kernels
     bool vec;
     Loop(const grav_plan* plan, int iters, void* work) : k(work_of(plan, iters)) {
-        unsigned char* b = (unsigned char*)work;
+        unsigned char* b = (unsigned char*)work + Work::kHead;
+        status = (int*)work;
         auto take = [&](size_t n) {
             R* v = (R*)b;
             b += n;
@@ -324,6 +338,7 @@ int run_start(grav_plan* plan, const R* d, const R* w, const R* wm, int iters, v
     const Loop<R> L(plan, iters, work);
     constexpr int V = 16 / sizeof(R);
     cudaError_t e = cudaMemsetAsync(L.pp, 0, L.k.dots() * sizeof(Dot), s);  // no block done yet
+    if (e == cudaSuccess) e = cudaMemsetAsync(L.status, 0, sizeof(int), s);
     if (e != cudaSuccess) return cuda_fail(e, "grav_cgls_start");
     cgls_first_data<R><<<L.gd, kVecThreads, 0, s>>>(d, w, L.r, L.wr, L.k.nd, L.rr(0));
     const int rc = grav_adjoint(plan, L.wr, L.g, s);
@@ -348,7 +363,7 @@ int run_steps(grav_plan* plan, const R* w, const R* wm, double lam, int iters, i
         int rc = grav_forward(plan, L.t, L.q, s);
         if (rc != GRAV_OK) return rc;
         cgls_weigh<R><<<L.gd, kVecThreads, 0, s>>>(w, L.q, L.k.nd, L.qq);
-        const Scalars k{L.ss(it), L.pp, L.qq, lam};
+        const Scalars k{L.ss(it), L.pp, L.qq, lam, L.status};
         cgls_step_data<R><<<L.gd, kVecThreads, 0, s>>>(k, w, L.q, L.r, L.wr, L.k.nd, L.rr(it + 1));
         rc = grav_adjoint(plan, L.wr, L.g, s);
         if (rc != GRAV_OK) return rc;

@@ -26,6 +26,7 @@ device operations with FP64 reductions.
 """
 from __future__ import annotations
 
+import math
 from dataclasses import dataclass
 
 import torch
@@ -116,7 +117,8 @@ def _on_device(plan, d: torch.Tensor, w, lam) -> bool:
     below operation by operation."""
     return (type(plan) is Plan and not {"forward", "adjoint"} & vars(plan).keys()
             and type(d) is torch.Tensor and type(w) is torch.Tensor
-            and isinstance(lam, (int, float)) and d.device == plan.device == w.device
+            and isinstance(lam, (int, float)) and not isinstance(lam, bool)
+            and abs(lam) <= torch.finfo(plan.dtype).max and d.device == plan.device == w.device
             and d.dtype == plan.dtype == w.dtype and tuple(d.shape) == (plan.ncomp, plan.ny, plan.nx)
             and w.dim() <= 3 and all(a in (1, b) for a, b in zip(w.shape[::-1], d.shape[::-1]))
             and not (d.requires_grad or w.requires_grad))
@@ -144,6 +146,14 @@ def _cgls_on_device(plan: Plan, d, w, wm, lam: float, iters: int, keep_models: b
     e1.record(s)
     m = models[-1].clone() if keep else models[0]
     objectives = obj.tolist()
+    if not all(map(math.isfinite, objectives)):
+        # a step whose length cannot be formed is an error, as in the loop below
+        at = base - work.data_ptr()
+        status = int(work[at:at + 4].view(torch.int32))
+        if status == 1:
+            raise ZeroDivisionError("float division by zero")
+        if status == 2:
+            raise RuntimeError(f"step length past the range of {d.dtype}")
     torch.cuda.synchronize()
     return CGLSResult(m=m, models=list(models.unbind(0)) if keep else [], objectives=objectives,
                       iterations=iters, lam=lam, ms_per_iteration=e0.elapsed_time(e1) / max(1, iters))

@@ -48,3 +48,16 @@ def test_fp32_loop_matches_the_stepwise_loop(gravlib, size):
     d = torch.empty((2, size[1], size[0]), device="cuda").normal_(generator=gen) * sigma * 50
     with Plan(mesh, comps) as a, StepwisePlan(mesh, comps) as b:
         assert_same(cgls(a, d, 1.0 / sigma, 1.0, iters=3), cgls(b, d, 1.0 / sigma, 1.0, iters=3))
+
+
+# (q, q) below FP32's range with data in SI units and no weights; a product of scale 1e-20, whose step is 1e40
+@pytest.mark.parametrize("scale,data,error", [(None, 1e-9, ZeroDivisionError), (1e-20, 1e19, RuntimeError)])
+def test_a_step_without_a_length_is_an_error(gravlib, scale, data, error):
+    mesh = (8, 8, 1, 20.0, 25.0, 15.0, 2000.0 if scale else 8.0)
+    comps = capi.GRAV_GZ if scale else capi.GRAV_GZZ
+    for cls in (Plan, StepwisePlan):
+        with cls(mesh, comps) as plan:
+            w = scale / float(plan.forward(torch.ones(1, 8, 8, device="cuda")).mean()) if scale else 1.0
+            weights = torch.full((1, 1, 1), w, device="cuda")
+            with pytest.raises(error):
+                cgls(plan, torch.full((1, 8, 8), data / w, device="cuda"), weights, 0.0, iters=2)
