@@ -192,6 +192,11 @@ int grav_cgls_start(grav_plan* plan, const void* d_dev, const void* w_dev, const
                     void* work_dev, void* stream);
 int grav_cgls_steps(grav_plan* plan, const void* w_dev, const void* wm_dev, double lam, int iters, int keep_models,
                     void* models_dev, double* objectives_dev, void* work_dev, void* stream);
+/* grav_cgls_steps that keeps the model after every step, each in a buffer of its
+ * own: models_dev is a host array of iters device pointers to [nz][ny][nx],
+ * 16-byte aligned, read before the call returns. */
+int grav_cgls_steps_kept(grav_plan* plan, const void* w_dev, const void* wm_dev, double lam, int iters,
+                         void* const* models_dev, double* objectives_dev, void* work_dev, void* stream);
 
 /* Release the plan and its device memory (waits for the device first).
  * NULL is ignored. */

@@ -51,6 +51,7 @@ EXPORTED = (
     "grav_cgls_work_bytes",
     "grav_cgls_start",
     "grav_cgls_steps",
+    "grav_cgls_steps_kept",
 )
 
 
@@ -135,6 +136,8 @@ def lib() -> ctypes.CDLL:
             L.grav_cgls_start.restype = i
             L.grav_cgls_steps.argtypes = [p, p, p, d, i, i, p, p, p, p]
             L.grav_cgls_steps.restype = i
+            L.grav_cgls_steps_kept.argtypes = [p, p, p, d, i, p, p, p, p]
+            L.grav_cgls_steps_kept.restype = i
             _lib = L
     return _lib
 
@@ -286,3 +289,10 @@ def grav_cgls_start(plan, d_ptr, w_ptr, wm_ptr, iters, work_ptr, stream=0) -> in
 def grav_cgls_steps(plan, w_ptr, wm_ptr, lam, iters, keep_models, models_ptr, objectives_ptr, work_ptr, stream=0) -> int:
     return _check(lib().grav_cgls_steps(plan, w_ptr, wm_ptr, float(lam), int(iters), 1 if keep_models else 0,
                                         models_ptr or None, objectives_ptr, work_ptr, stream or None))
+
+
+def grav_cgls_steps_kept(plan, w_ptr, wm_ptr, lam, model_ptrs, objectives_ptr, work_ptr, stream=0) -> int:
+    """One step per entry of model_ptrs, which receives that step's model."""
+    arr = (ctypes.c_void_p * len(model_ptrs))(*model_ptrs)
+    return _check(lib().grav_cgls_steps_kept(plan, w_ptr, wm_ptr, float(lam), len(model_ptrs), arr, objectives_ptr,
+                                             work_ptr, stream or None))

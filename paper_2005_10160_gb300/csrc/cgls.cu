@@ -333,6 +333,13 @@ template <typename R> struct Loop {
     Dot* ss(int it) const { return rr(it) + 2; }
 };
 
+// Where the steps leave models: one buffer per step (host array of device
+// pointers), the steps' models in one block, or the last step's model only.
+template <typename R> struct Models {
+    void* const* each;
+    R *block, *last;
+};
+
 template <typename R>
 int run_start(grav_plan* plan, const R* d, const R* w, const R* wm, int iters, void* work, cudaStream_t s) {
     const Loop<R> L(plan, iters, work);
@@ -350,13 +357,13 @@ int run_start(grav_plan* plan, const R* d, const R* w, const R* wm, int iters, v
 }
 
 template <typename R>
-int run_steps(grav_plan* plan, const R* w, const R* wm, double lam, int iters, int keep, R* models, double* obj,
+int run_steps(grav_plan* plan, const R* w, const R* wm, double lam, int iters, const Models<R>& models, double* obj,
               void* work, cudaStream_t s) {
     const Loop<R> L(plan, iters, work);
     constexpr int V = 16 / sizeof(R);
     const size_t cells = L.k.plane * L.k.nz;
-    if (iters == 0 && !keep) {
-        const cudaError_t e = cudaMemsetAsync(models, 0, cells * sizeof(R), s);
+    if (iters == 0 && models.last) {
+        const cudaError_t e = cudaMemsetAsync(models.last, 0, cells * sizeof(R), s);
         if (e != cudaSuccess) return cuda_fail(e, "grav_cgls_steps");
     }
     for (int it = 0; it < iters; ++it) {
@@ -367,7 +374,7 @@ int run_steps(grav_plan* plan, const R* w, const R* wm, double lam, int iters, i
         cgls_step_data<R><<<L.gd, kVecThreads, 0, s>>>(k, w, L.q, L.r, L.wr, L.k.nd, L.rr(it + 1));
         rc = grav_adjoint(plan, L.wr, L.g, s);
         if (rc != GRAV_OK) return rc;
-        R* m = keep ? models + (size_t)it * cells : it + 1 == iters ? models : nullptr;
+        R* m = models.each ? (R*)models.each[it] : models.block ? models.block + it * cells : it + 1 == iters ? models.last : nullptr;
         if (L.vec) cgls_step_model<R, V><<<L.gm, kVecThreads, 0, s>>>(k, it == 0, wm, L.p, L.x, L.g, m, L.k.plane, L.k.nz, L.ss(it + 1), L.xx(it + 1));
         else cgls_step_model<R, 1><<<L.gm, kVecThreads, 0, s>>>(k, it == 0, wm, L.p, L.x, L.g, m, L.k.plane, L.k.nz, L.ss(it + 1), L.xx(it + 1));
         if (it + 1 < iters) {
@@ -396,6 +403,27 @@ int check_cgls(const grav_plan* plan, bool pointers, int iters, const void* work
     return GRAV_OK;
 }
 
+int steps(grav_plan* plan, const void* w, const void* wm, double lam, int iters, void* const* each, void* block,
+          void* last, double* obj, void* work, cudaStream_t s, const char* name) {
+    uintptr_t bits = reinterpret_cast<uintptr_t>(block) | reinterpret_cast<uintptr_t>(last);
+    for (int it = 0; each && it < iters; ++it) {
+        if (!each[it]) {
+            set_error("%s: null model buffer", name);
+            return GRAV_EINVAL;
+        }
+        bits |= reinterpret_cast<uintptr_t>(each[it]);
+    }
+    if (bits & 15) {
+        set_error("%s: models must be 16-byte aligned", name);
+        return GRAV_EINVAL;
+    }
+    if (plan->fp64)
+        return run_steps<double>(plan, (const double*)w, (const double*)wm, lam, iters,
+                                 Models<double>{each, (double*)block, (double*)last}, obj, work, s);
+    return run_steps<float>(plan, (const float*)w, (const float*)wm, lam, iters,
+                            Models<float>{each, (float*)block, (float*)last}, obj, work, s);
+}
+
 }  // namespace
 
 }  // namespace grav
@@ -422,15 +450,17 @@ int grav_cgls_steps(grav_plan* plan, const void* w_dev, const void* wm_dev, doub
     const int rc = check_cgls(plan, w_dev && wm_dev && objectives_dev && (models_dev || (keep_models && iters == 0)), iters,
                               work_dev, "grav_cgls_steps");
     if (rc != GRAV_OK) return rc;
-    if (reinterpret_cast<uintptr_t>(models_dev) & 15) {
-        set_error("grav_cgls_steps: models must be 16-byte aligned");
-        return GRAV_EINVAL;
-    }
-    cudaStream_t s = (cudaStream_t)stream;
-    return plan->fp64 ? run_steps<double>(plan, (const double*)w_dev, (const double*)wm_dev, lam, iters, keep_models,
-                                          (double*)models_dev, objectives_dev, work_dev, s)
-                      : run_steps<float>(plan, (const float*)w_dev, (const float*)wm_dev, lam, iters, keep_models,
-                                         (float*)models_dev, objectives_dev, work_dev, s);
+    return steps(plan, w_dev, wm_dev, lam, iters, nullptr, keep_models ? models_dev : nullptr,
+                 keep_models ? nullptr : models_dev, objectives_dev, work_dev, (cudaStream_t)stream, "grav_cgls_steps");
+}
+
+int grav_cgls_steps_kept(grav_plan* plan, const void* w_dev, const void* wm_dev, double lam, int iters,
+                         void* const* models_dev, double* objectives_dev, void* work_dev, void* stream) {
+    const int rc = check_cgls(plan, w_dev && wm_dev && objectives_dev && (models_dev || iters == 0), iters, work_dev,
+                              "grav_cgls_steps_kept");
+    if (rc != GRAV_OK) return rc;
+    return steps(plan, w_dev, wm_dev, lam, iters, models_dev, nullptr, nullptr, objectives_dev, work_dev,
+                 (cudaStream_t)stream, "grav_cgls_steps_kept");
 }
 
 }  // extern "C"

@@ -135,14 +135,18 @@ def _cgls_on_device(plan: Plan, d, w, wm, lam: float, iters: int, keep_models: b
     work = torch.empty(capi.grav_cgls_work_bytes(plan.handle, n) + 256, dtype=torch.uint8, device=d.device)
     base = (work.data_ptr() + 255) // 256 * 256
     keep = keep_models and n > 0
-    models = torch.empty((n if keep else 1, nz, ny, nx), dtype=d.dtype, device=d.device)
+    models = [torch.empty((nz, ny, nx), dtype=d.dtype, device=d.device) for _ in range(n if keep else 1)]
     obj = torch.empty(n + 1, dtype=torch.float64, device=d.device)
     s = torch.cuda.current_stream(d.device)
     e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     capi.grav_cgls_start(plan.handle, d.data_ptr(), w.data_ptr(), wm1.data_ptr(), n, base, s.cuda_stream)
     e0.record(s)
-    capi.grav_cgls_steps(plan.handle, w.data_ptr(), wm1.data_ptr(), lam, n, keep, models.data_ptr(), obj.data_ptr(), base,
-                         s.cuda_stream)
+    if keep:
+        capi.grav_cgls_steps_kept(plan.handle, w.data_ptr(), wm1.data_ptr(), lam, [m.data_ptr() for m in models],
+                                  obj.data_ptr(), base, s.cuda_stream)
+    else:
+        capi.grav_cgls_steps(plan.handle, w.data_ptr(), wm1.data_ptr(), lam, n, False, models[0].data_ptr(),
+                             obj.data_ptr(), base, s.cuda_stream)
     e1.record(s)
     m = models[-1].clone() if keep else models[0]
     objectives = obj.tolist()
@@ -155,7 +159,7 @@ def _cgls_on_device(plan: Plan, d, w, wm, lam: float, iters: int, keep_models: b
         if status == 2:
             raise RuntimeError(f"step length past the range of {d.dtype}")
     torch.cuda.synchronize()
-    return CGLSResult(m=m, models=list(models.unbind(0)) if keep else [], objectives=objectives,
+    return CGLSResult(m=m, models=models if keep else [], objectives=objectives,
                       iterations=iters, lam=lam, ms_per_iteration=e0.elapsed_time(e1) / max(1, iters))
 
 

@@ -1,5 +1,6 @@
-"""FP32 sums of squares of the inversion loop enqueued by the library, against
-the loop operation by operation (a plan subclass takes that path).
+"""The inversion loop enqueued by the library, against the loop operation by
+operation (a plan subclass takes that path): FP32 sums of squares, steps that
+have no length, kept models.
 
 Bar 1e-3: the two differ in the rounding of FP32 vector updates, 2^-24, which CG
 amplifies about 1e4 times within eight steps (the FP64 loops differ by 1e-12)."""
@@ -61,3 +62,16 @@ def test_a_step_without_a_length_is_an_error(gravlib, scale, data, error):
             weights = torch.full((1, 1, 1), w, device="cuda")
             with pytest.raises(error):
                 cgls(plan, torch.full((1, 8, 8), data / w, device="cuda"), weights, 0.0, iters=2)
+
+
+def test_kept_models_have_memory_of_their_own(gravlib):
+    """Keeping one model must not keep the others alive."""
+    mesh = (12, 10, 3, 20.0, 25.0, 15.0, 8.0)
+    gen = torch.Generator(device="cuda").manual_seed(1)
+    d = torch.empty((1, 10, 12), device="cuda").normal_(generator=gen) * 5e-5
+    with Plan(mesh, capi.GRAV_GZ) as plan:
+        res = cgls(plan, d, torch.full((1, 1, 1), 1e6, device="cuda"), 1.0, iters=3, keep_models=True)
+    stores = [m.untyped_storage() for m in (*res.models, res.m)]
+    assert len({s.data_ptr() for s in stores}) == 4
+    assert all(s.nbytes() == m.numel() * m.element_size() for s, m in zip(stores, (*res.models, res.m)))
+    assert torch.equal(res.models[-1], res.m)
