@@ -50,22 +50,28 @@ __device__ __forceinline__ double block_sum(double v) {
     return s;
 }
 
-// A dot product in the making: one partial per block, the number of blocks
-// done (0 before and after each use), and the result.
+// A dot product: the result, and the number of blocks that have handed in
+// their share (0 before and after each use).
 struct Dot {
     double value;
     unsigned done, pad;
-    double parts[kMaxParts];
+};
+// A dot product in the making and where the blocks' partials go: one array per
+// dot product of a kernel, free again when the kernel ends.
+struct Making {
+    Dot* dot;
+    double* parts;
 };
 
 // Every block of the grid hands in its share (all threads call this); the last
 // one adds the partials up in block order.
-__device__ __forceinline__ void put_dot(Dot* d, double share) {
+__device__ __forceinline__ void put_dot(Making m, double share) {
+    Dot* d = m.dot;
     __shared__ bool last;
     const unsigned nb = gridDim.x * gridDim.y, b = blockIdx.y * gridDim.x + blockIdx.x;
     const double s = block_sum(share);
     if (threadIdx.x == 0) {
-        d->parts[b] = s;
+        m.parts[b] = s;
         __threadfence();
         last = atomicInc(&d->done, nb - 1) == nb - 1;  // wraps to 0 for the next use
     }
@@ -73,7 +79,7 @@ __device__ __forceinline__ void put_dot(Dot* d, double share) {
     if (!last) return;
     __threadfence();
     double v = 0.0;
-    for (unsigned i = threadIdx.x; i < nb; i += kVecThreads) v += __ldcg(&d->parts[i]);
+    for (unsigned i = threadIdx.x; i < nb; i += kVecThreads) v += __ldcg(&m.parts[i]);
     v = block_sum(v);
     if (threadIdx.x == 0) d->value = v;
 }
@@ -131,7 +137,7 @@ __device__ __forceinline__ double step_length(const Scalars& k) {
 // r = w d, wr = w r, (r, r)
 template <typename R>
 __global__ void __launch_bounds__(kVecThreads) cgls_first_data(const R* __restrict__ d, const R* __restrict__ w, R* __restrict__ r,
-                                                               R* __restrict__ wr, size_t n, Dot* rr) {
+                                                               R* __restrict__ wr, size_t n, Making rr) {
     Squares<R> s;
     for (size_t i = (size_t)blockIdx.x * kVecThreads + threadIdx.x; i < n; i += (size_t)gridDim.x * kVecThreads) {
         const R v = w[i] * d[i];
@@ -144,7 +150,7 @@ __global__ void __launch_bounds__(kVecThreads) cgls_first_data(const R* __restri
 
 // q = w y in place, (q, q)
 template <typename R>
-__global__ void __launch_bounds__(kVecThreads) cgls_weigh(const R* __restrict__ w, R* __restrict__ q, size_t n, Dot* qq) {
+__global__ void __launch_bounds__(kVecThreads) cgls_weigh(const R* __restrict__ w, R* __restrict__ q, size_t n, Making qq) {
     Squares<R> s;
     for (size_t i = (size_t)blockIdx.x * kVecThreads + threadIdx.x; i < n; i += (size_t)gridDim.x * kVecThreads) {
         const R v = w[i] * q[i];
@@ -158,7 +164,7 @@ __global__ void __launch_bounds__(kVecThreads) cgls_weigh(const R* __restrict__ 
 // but (q, q) + lam (p, p) = 0) or with one past R's range
 template <typename R>
 __global__ void __launch_bounds__(kVecThreads) cgls_step_data(Scalars k, const R* __restrict__ w, const R* __restrict__ q, R* __restrict__ r,
-                                                              R* __restrict__ wr, size_t n, Dot* rr) {
+                                                              R* __restrict__ wr, size_t n, Making rr) {
     const double step = step_length(k);
     const R alpha = (R)step;
     if (blockIdx.x == 0 && threadIdx.x == 0 && *k.status == kStepsDone) {
@@ -186,7 +192,7 @@ __global__ void __launch_bounds__(kVecThreads) cgls_step_data(Scalars k, const R
 // s = g / w_n in place, p = s, t = p / w_n, (s, s)
 template <typename R, int VEC>
 __global__ void __launch_bounds__(kVecThreads) cgls_first_model(const R* __restrict__ wm, R* __restrict__ g, R* __restrict__ p,
-                                                                R* __restrict__ t, size_t plane, int nz, Dot* ss, Dot* pp) {
+                                                                R* __restrict__ t, size_t plane, int nz, Making ss, Making pp) {
     using P = Pack<R, VEC>;
     Squares<R> sum;
     GRAV_FOR_LAYERS
@@ -211,7 +217,7 @@ __global__ void __launch_bounds__(kVecThreads) cgls_first_model(const R* __restr
 template <typename R, int VEC>
 __global__ void __launch_bounds__(kVecThreads) cgls_step_model(Scalars k, bool first, const R* __restrict__ wm, const R* __restrict__ p, R* __restrict__ x,
                                                                R* __restrict__ g, R* __restrict__ m, size_t plane, int nz,
-                                                               Dot* ss, Dot* xx) {
+                                                               Making ss, Making xx) {
     using P = Pack<R, VEC>;
     const R alpha = (R)step_length(k), lam = (R)k.lam;
     Squares<R> s2, x2;
@@ -246,7 +252,7 @@ __global__ void __launch_bounds__(kVecThreads) cgls_step_model(Scalars k, bool f
 template <typename R, int VEC>
 __global__ void __launch_bounds__(kVecThreads) cgls_next_dir(const Dot* gamma, const Dot* gamma_new, const R* __restrict__ wm,
                                                              const R* __restrict__ s, R* __restrict__ p, R* __restrict__ t,
-                                                             size_t plane, int nz, Dot* pp) {
+                                                             size_t plane, int nz, Making pp) {
     using P = Pack<R, VEC>;
     __shared__ double beta_sh;
     if (threadIdx.x == 0) beta_sh = gamma->value == 0.0 ? 0.0 : gamma_new->value / gamma->value;
@@ -278,14 +284,15 @@ __global__ void __launch_bounds__(kVecThreads) cgls_objectives(const Dot* dots, 
 size_t pad256(size_t v) { return (v + 255) / 256 * 256; }
 
 // The caller's workspace: the status; data vectors r, q, wr; model vectors p, t,
-// g, x; then the dot products: (p, p), (q, q) and, per step, (r, r), (x, x),
-// (s, s).
+// g, x; two arrays of partials; then the dot products: (p, p), (q, q) and, per
+// step, (r, r), (x, x), (s, s).
 struct Work {
     static constexpr size_t kHead = 256;  // the status
     size_t nd, plane, data, model;
     int nz, iters;
     size_t dots() const { return 2 + 3 * ((size_t)iters + 1); }
-    size_t bytes() const { return kHead + 3 * data + 4 * model + dots() * sizeof(Dot); }
+    static constexpr size_t kParts = kMaxParts * sizeof(double);
+    size_t bytes() const { return kHead + 3 * data + 4 * model + 2 * kParts + dots() * sizeof(Dot); }
 };
 Work work_of(const grav_plan* p, int iters) {
     Work w{};
@@ -303,6 +310,7 @@ template <typename R> struct Loop {
     Work k;
     int* status;
     R *r, *q, *wr, *p, *t, *g, *x;
+    double* parts;
     Dot *pp, *qq, *step;
     unsigned gd;      // blocks of the data-size kernels
     dim3 gm;          // blocks of the model-size kernels
@@ -317,7 +325,8 @@ template <typename R> struct Loop {
         };
         r = take(k.data), q = take(k.data), wr = take(k.data);
         p = take(k.model), t = take(k.model), g = take(k.model), x = take(k.model);
-        pp = (Dot*)b;
+        parts = (double*)b;
+        pp = (Dot*)(b + 2 * Work::kParts);
         qq = pp + 1;
         step = pp + 2;
         gd = (unsigned)std::min<size_t>((k.nd + kVecThreads - 1) / kVecThreads, kMaxParts / 2);
@@ -328,6 +337,8 @@ template <typename R> struct Loop {
         const unsigned gx = (unsigned)std::min<size_t>((k.plane + per - 1) / per, kMaxParts / gy);
         gm = dim3(gx, gy);
     }
+    Making first(Dot* d) const { return {d, parts}; }
+    Making second(Dot* d) const { return {d, parts + kMaxParts}; }
     Dot* rr(int it) const { return step + (size_t)3 * it; }
     Dot* xx(int it) const { return rr(it) + 1; }
     Dot* ss(int it) const { return rr(it) + 2; }
@@ -347,11 +358,11 @@ int run_start(grav_plan* plan, const R* d, const R* w, const R* wm, int iters, v
     cudaError_t e = cudaMemsetAsync(L.pp, 0, L.k.dots() * sizeof(Dot), s);  // no block done yet
     if (e == cudaSuccess) e = cudaMemsetAsync(L.status, 0, sizeof(int), s);
     if (e != cudaSuccess) return cuda_fail(e, "grav_cgls_start");
-    cgls_first_data<R><<<L.gd, kVecThreads, 0, s>>>(d, w, L.r, L.wr, L.k.nd, L.rr(0));
+    cgls_first_data<R><<<L.gd, kVecThreads, 0, s>>>(d, w, L.r, L.wr, L.k.nd, L.first(L.rr(0)));
     const int rc = grav_adjoint(plan, L.wr, L.g, s);
     if (rc != GRAV_OK) return rc;
-    if (L.vec) cgls_first_model<R, V><<<L.gm, kVecThreads, 0, s>>>(wm, L.g, L.p, L.t, L.k.plane, L.k.nz, L.ss(0), L.pp);
-    else cgls_first_model<R, 1><<<L.gm, kVecThreads, 0, s>>>(wm, L.g, L.p, L.t, L.k.plane, L.k.nz, L.ss(0), L.pp);
+    if (L.vec) cgls_first_model<R, V><<<L.gm, kVecThreads, 0, s>>>(wm, L.g, L.p, L.t, L.k.plane, L.k.nz, L.first(L.ss(0)), L.second(L.pp));
+    else cgls_first_model<R, 1><<<L.gm, kVecThreads, 0, s>>>(wm, L.g, L.p, L.t, L.k.plane, L.k.nz, L.first(L.ss(0)), L.second(L.pp));
     e = cudaGetLastError();
     return e == cudaSuccess ? GRAV_OK : cuda_fail(e, "grav_cgls_start");
 }
@@ -369,17 +380,17 @@ int run_steps(grav_plan* plan, const R* w, const R* wm, double lam, int iters, c
     for (int it = 0; it < iters; ++it) {
         int rc = grav_forward(plan, L.t, L.q, s);
         if (rc != GRAV_OK) return rc;
-        cgls_weigh<R><<<L.gd, kVecThreads, 0, s>>>(w, L.q, L.k.nd, L.qq);
+        cgls_weigh<R><<<L.gd, kVecThreads, 0, s>>>(w, L.q, L.k.nd, L.first(L.qq));
         const Scalars k{L.ss(it), L.pp, L.qq, lam, L.status};
-        cgls_step_data<R><<<L.gd, kVecThreads, 0, s>>>(k, w, L.q, L.r, L.wr, L.k.nd, L.rr(it + 1));
+        cgls_step_data<R><<<L.gd, kVecThreads, 0, s>>>(k, w, L.q, L.r, L.wr, L.k.nd, L.first(L.rr(it + 1)));
         rc = grav_adjoint(plan, L.wr, L.g, s);
         if (rc != GRAV_OK) return rc;
         R* m = models.each ? (R*)models.each[it] : models.block ? models.block + it * cells : it + 1 == iters ? models.last : nullptr;
-        if (L.vec) cgls_step_model<R, V><<<L.gm, kVecThreads, 0, s>>>(k, it == 0, wm, L.p, L.x, L.g, m, L.k.plane, L.k.nz, L.ss(it + 1), L.xx(it + 1));
-        else cgls_step_model<R, 1><<<L.gm, kVecThreads, 0, s>>>(k, it == 0, wm, L.p, L.x, L.g, m, L.k.plane, L.k.nz, L.ss(it + 1), L.xx(it + 1));
+        if (L.vec) cgls_step_model<R, V><<<L.gm, kVecThreads, 0, s>>>(k, it == 0, wm, L.p, L.x, L.g, m, L.k.plane, L.k.nz, L.first(L.ss(it + 1)), L.second(L.xx(it + 1)));
+        else cgls_step_model<R, 1><<<L.gm, kVecThreads, 0, s>>>(k, it == 0, wm, L.p, L.x, L.g, m, L.k.plane, L.k.nz, L.first(L.ss(it + 1)), L.second(L.xx(it + 1)));
         if (it + 1 < iters) {
-            if (L.vec) cgls_next_dir<R, V><<<L.gm, kVecThreads, 0, s>>>(L.ss(it), L.ss(it + 1), wm, L.g, L.p, L.t, L.k.plane, L.k.nz, L.pp);
-            else cgls_next_dir<R, 1><<<L.gm, kVecThreads, 0, s>>>(L.ss(it), L.ss(it + 1), wm, L.g, L.p, L.t, L.k.plane, L.k.nz, L.pp);
+            if (L.vec) cgls_next_dir<R, V><<<L.gm, kVecThreads, 0, s>>>(L.ss(it), L.ss(it + 1), wm, L.g, L.p, L.t, L.k.plane, L.k.nz, L.first(L.pp));
+            else cgls_next_dir<R, 1><<<L.gm, kVecThreads, 0, s>>>(L.ss(it), L.ss(it + 1), wm, L.g, L.p, L.t, L.k.plane, L.k.nz, L.first(L.pp));
         }
     }
     cgls_objectives<<<1, kVecThreads, 0, s>>>(L.step, iters + 1, lam, obj);

@@ -1,6 +1,6 @@
 """The inversion loop enqueued by the library, against the loop operation by
 operation (a plan subclass takes that path): FP32 sums of squares, steps that
-have no length, kept models.
+have no length, kept models, workspace.
 
 Bar 1e-3: the two differ in the rounding of FP32 vector updates, 2^-24, which CG
 amplifies about 1e4 times within eight steps (the FP64 loops differ by 1e-12)."""
@@ -75,3 +75,9 @@ def test_kept_models_have_memory_of_their_own(gravlib):
     assert len({s.data_ptr() for s in stores}) == 4
     assert all(s.nbytes() == m.numel() * m.element_size() for s, m in zip(stores, (*res.models, res.m)))
     assert torch.equal(res.models[-1], res.m)
+
+
+def test_workspace_of_a_long_loop(gravlib):
+    """A step adds three dot products of 16 bytes to the workspace."""
+    with Plan((12, 10, 3, 20.0, 25.0, 15.0, 8.0), capi.GRAV_GZ) as plan:
+        assert capi.grav_cgls_work_bytes(plan.handle, 1001) - capi.grav_cgls_work_bytes(plan.handle, 1) == 1000 * 48
