@@ -213,7 +213,7 @@ int make_spectra(grav_plan* p) {
         } else {
             const Geometry g{p->nx, p->ny, p->nz, p->dx, p->dy, p->dz, p->h};
             SpecBuild b{p->nx, p->ny, p->nz, ny2, p->ncomp, p->kx_count, p->jp, p->log_px, p->log_py, 0, p->oddv_mask};
-            GenOut o = gen_out(p->fp64 ? GenOut::kQuadrant : GenOut::kQuadrantPairs, !p->fp64);
+            GenOut o = gen_out(p->fp64 ? GenOut::kQuadrant : GenOut::kQuadrantPairs, !p->fp64 && corner_tables_fit(g));
             double factor[kMaxPlanComp];
             // FP32 pairs: kernels in units of upsilon (times the largest cell
             // edge for first derivatives), which are of order 1 at most

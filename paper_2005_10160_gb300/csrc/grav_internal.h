@@ -200,9 +200,13 @@ struct GenOut {
     };
     Mode mode;
     bool tables;             // the faster corner terms, for values that end up in FP32 spectra
+                             // (plane plans: where corner_tables_fit)
     int px, py;              // kHalfRows
     double factor[kMaxComp];  // value = factor[component] times the corner sum (upsilon for SI units)
 };
+// Whether the rounding of the faster corner terms stays far below FP32's in the
+// fields of a plane plan.
+bool corner_tables_fit(const Geometry& g);
 // Output of the given mode in SI units.
 GenOut gen_out(GenOut::Mode mode, bool tables, int px = 0, int py = 0);
 // Layers n0 .. n1 (nzc = n1 - n0), one slot per selected component.

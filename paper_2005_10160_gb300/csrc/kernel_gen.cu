@@ -53,11 +53,9 @@ __device__ __forceinline__ Dist distance(double a, double b) {
 // without gx, gy use 7 so that the kernel keeps fewer registers.  rxy, rxz,
 // ryz: distances in the coordinate planes.
 //
-// TABLES (plans that store FP32 spectra): corner_terms.cuh and the shared
-// distances, whose rounding is up to 1.23 times that of the other form for
-// some components (0.87 to 0.95 for gz), far below FP32's.  Otherwise (FP64
-// plans, kernel values) CUDA's asinh and atan, 2.3 times the FP64
-// instructions.
+// TABLES: corner_terms.cuh and the shared distances, for plans that store FP32
+// spectra (see corner_tables_fit).  Otherwise CUDA's asinh and atan, 2.3 times
+// the FP64 instructions.
 template <int NC, bool TABLES>
 __device__ __forceinline__ void corner_terms(double x, double y, double z, const Dist* rxy, const Dist* rxz,
                                              const Dist* ryz, unsigned comps, const CornerTables& t,
@@ -241,6 +239,26 @@ cudaError_t launch_kernel_gen(const Geometry& g, const GenOut& o, unsigned comps
     if (o.tables)
         return nine ? gen_launch<9, true>(g, o, comps, n0, n1, out, s) : gen_launch<7, true>(g, o, comps, n0, n1, out, s);
     return nine ? gen_launch<9, false>(g, o, comps, n0, n1, out, s) : gen_launch<7, false>(g, o, comps, n0, n1, out, s);
+}
+
+// The eight corner terms cancel, so a kernel value carries their rounding
+// enlarged.  Over meshes wider than they are deep that stays below FP32's
+// rounding in the field, and the tables' is 0.7 .. 1.2 times the library
+// functions'.  For a narrow mesh far below its stations it does not: with z the
+// deepest level, V a cell's volume and X, Y the mesh's width it is about 2^-53
+// z^3 / V, times z / X and z / Y for the components odd in x and y, and the
+// tables' rounding of those is up to 2.3 times the functions' (7 x 3 x 5 cells
+// of 84 x 40 x 65 m at 6800 m: gxy 4.3e-7 of the field with the functions, 1e-6
+// with the tables).  Measured on 220 meshes of 3 .. 1024 cells a side, both
+// layers' ends and nine components against 113-bit arithmetic: what the tables
+// add to a field error of 2e-7 is below 3e-4 of it up to a factor of 2^22, and
+// below 2e-4 of it on every mesh no deeper than wide.  (Equal-dimension plans
+// transform all depths together, where the offsets near a station set the
+// size: they always take the tables for FP32 spectra.)
+bool corner_tables_fit(const Geometry& g) {
+    const double z = g.h + g.nz * g.dz, X = std::max(g.nx - 1, 1) * g.dx, Y = std::max(g.ny - 1, 1) * g.dy;
+    if (z <= X && z <= Y) return true;
+    return z / g.dx * (z / g.dy) * (z / g.dz) * std::max(1.0, z / X) * std::max(1.0, z / Y) <= 0x1p22;
 }
 
 GenOut gen_out(GenOut::Mode mode, bool tables, int px, int py) {
