@@ -23,9 +23,11 @@
 // an FP32 plan's sum as an unevaluated pair of floats: the product's rounding
 // error by fused multiply-add, the sum's by the two-sum of Knuth (TAOCP 2,
 // 4.2.2), both added to the low part; the sum is good to about 2^-45, more than
-// that of separately rounded FP32 products.  A pair has FP32's range: sums from
-// 2^100 on move to an FP64 number, and the rounding error of a square below
-// about 1e-32 is lost, as in an FP32 product.
+// that of separately rounded FP32 products.  A pair has FP32's range: a thread
+// whose sum leaves it adds FP32 products in FP64 over the values it has stored
+// (a test for it in the loop, with FP64 instructions behind it, took the three
+// iterations below from 2.08 to 3.06 ms), and the rounding error of a square
+// below about 1e-32 is lost, as in an FP32 product.
 #include <algorithm>
 
 #include "grav_internal.h"
@@ -89,29 +91,39 @@ template <typename R> struct Squares;
 template <> struct Squares<double> {
     double s = 0.0;
     __device__ __forceinline__ void add(double v) { s += v * v; }
-    __device__ __forceinline__ double get() const { return s; }
+    template <typename F> __device__ __forceinline__ double get(F&&) const { return s; }
 };
 template <> struct Squares<float> {
     float hi = 0.f, lo = 0.f;
-    double big = 0.0;
     __device__ __forceinline__ void add(float v) {
         const float p = __fmul_rn(v, v), pe = __fmaf_rn(v, v, -p);
         const float t = __fadd_rn(hi, p), z = __fsub_rn(t, hi);
         const float te = __fadd_rn(__fsub_rn(hi, __fsub_rn(t, z)), __fsub_rn(p, z));
         hi = t;
         lo = __fadd_rn(lo, __fadd_rn(pe, te));
-        // a finite square added to less than 2^100 stays finite
-        if (hi >= 0x1p100f) {
-            big += pair();
-            hi = lo = 0.f;
-        }
     }
-    // past the FP32 range (an infinite square) the corrections are not numbers; the sum is
-    __device__ __forceinline__ double pair() const { return isfinite(lo) ? (double)hi + (double)lo : (double)hi; }
-    __device__ __forceinline__ double get() const { return big + pair(); }
+    // again(f) calls f with every value once more
+    template <typename F> __device__ __forceinline__ double get(F&& again) const {
+        if (isfinite(hi)) return (double)hi + (double)lo;
+        double s = 0.0;
+        again([&](float v) { s += (double)__fmul_rn(v, v); });
+        return s;
+    }
 };
 
 template <typename R, int VEC> struct alignas(sizeof(R) * VEC) Pack { R v[VEC]; };
+
+// f(v) for every value of a data-size vector that this thread wrote.
+template <typename R, typename F> __device__ __forceinline__ void each_data(const R* v, size_t n, F&& f) {
+    for (size_t i = (size_t)blockIdx.x * kVecThreads + threadIdx.x; i < n; i += (size_t)gridDim.x * kVecThreads) f(v[i]);
+}
+// The same for a model-size vector.
+template <int VEC, typename R, typename F>
+__device__ __forceinline__ void each_model(const R* v, size_t plane, int nz, F&& f) {
+    for (int n = blockIdx.y; n < nz; n += gridDim.y)
+        for (size_t i = ((size_t)blockIdx.x * kVecThreads + threadIdx.x) * VEC; i < plane; i += (size_t)gridDim.x * kVecThreads * VEC)
+            for (int j = 0; j < VEC; ++j) f(v[(size_t)n * plane + i + j]);
+}
 
 // What the steps found, the first int of the workspace.
 enum { kStepsDone = 0, kNoStepLength = 1, kStepLengthRange = 2 };
@@ -145,7 +157,7 @@ __global__ void __launch_bounds__(kVecThreads) cgls_first_data(const R* __restri
         wr[i] = w[i] * v;
         s.add(v);
     }
-    put_dot(rr, s.get());
+    put_dot(rr, s.get([&](auto f) { each_data(r, n, f); }));
 }
 
 // q = w y in place, (q, q)
@@ -157,7 +169,7 @@ __global__ void __launch_bounds__(kVecThreads) cgls_weigh(const R* __restrict__ 
         q[i] = v;
         s.add(v);
     }
-    put_dot(qq, s.get());
+    put_dot(qq, s.get([&](auto f) { each_data(q, n, f); }));
 }
 
 // r -= alpha q, wr = w r, (r, r); records a step without a length (a gradient,
@@ -178,7 +190,7 @@ __global__ void __launch_bounds__(kVecThreads) cgls_step_data(Scalars k, const R
         wr[i] = w[i] * v;
         s.add(v);
     }
-    put_dot(rr, s.get());
+    put_dot(rr, s.get([&](auto f) { each_data(r, n, f); }));
 }
 
 // Model-size kernels: block rows take layers blockIdx.y, blockIdx.y + gridDim.y,
@@ -208,8 +220,9 @@ __global__ void __launch_bounds__(kVecThreads) cgls_first_model(const R* __restr
             *reinterpret_cast<P*>(t + base + i) = tv;
         }
     }
-    put_dot(ss, sum.get());
-    put_dot(pp, sum.get());
+    const double share = sum.get([&](auto f) { each_model<VEC>(p, plane, nz, f); });
+    put_dot(ss, share);
+    put_dot(pp, share);
 }
 
 // x += alpha p (x = alpha p in the first step), s = g / w_n - lam x in place
@@ -244,8 +257,8 @@ __global__ void __launch_bounds__(kVecThreads) cgls_step_model(Scalars k, bool f
             if (m) *reinterpret_cast<P*>(m + base + i) = mv;
         }
     }
-    put_dot(ss, s2.get());
-    put_dot(xx, x2.get());
+    put_dot(ss, s2.get([&](auto f) { each_model<VEC>(g, plane, nz, f); }));
+    put_dot(xx, x2.get([&](auto f) { each_model<VEC>(x, plane, nz, f); }));
 }
 
 // p = s + beta p, t = p / w_n, (p, p)
@@ -272,7 +285,7 @@ __global__ void __launch_bounds__(kVecThreads) cgls_next_dir(const Dot* gamma, c
             *reinterpret_cast<P*>(t + base + i) = tv;
         }
     }
-    put_dot(pp, p2.get());
+    put_dot(pp, p2.get([&](auto f) { each_model<VEC>(p, plane, nz, f); }));
 }
 #undef GRAV_FOR_LAYERS
 
