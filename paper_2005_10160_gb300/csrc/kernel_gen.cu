@@ -105,35 +105,36 @@ __device__ __forceinline__ float2 split_pair(double v) {
     return ok ? make_float2(__uint_as_float(hb), (float)(v - hd)) : make_float2((float)v, 0.f);
 }
 
-// Offsets per CTA: a kGenTX x kGenTY tile of the quadrant.  Neighbouring
+// Offsets per CTA: a kGenTX x TY tile of the quadrant.  Neighbouring
 // offsets share prism corners (the far x-corner of offset u is the near one
 // of u + 1), so the CTA evaluates the corner terms of its (kGenTX + 1) x
-// (kGenTY + 1) corners once per z-level, keeps the difference to the level
+// (TY + 1) corners once per z-level, keeps the difference to the level
 // above in shared memory, and every thread forms its offsets' kernel values
 // from four differences.  blockIdx.z takes a run of `per` layers.
 //
 // Bound by FP64 issue.  1024 x 1024 x 100, six components: 65 ms with the
 // tables, 92 ms with the library's asinh and atan and tiles of 32 x 8.
-constexpr int kGenTX = 32, kGenTY = 16, kGenThreads = 256;
-constexpr int kGenCX = kGenTX + 1, kGenCY = kGenTY + 1, kGenCor = kGenCX * kGenCY;
-constexpr size_t gen_smem(int nc) {
-    return sizeof(CornerTables) + (size_t)kGenCor * 2 * nc * sizeof(double) +
-           (size_t)(kGenCor + kGenCX + kGenCY) * sizeof(Dist);
-}
+constexpr int kGenTX = 32, kGenThreads = 256;
+template <int TY> struct GenTile {
+    static constexpr int CX = kGenTX + 1, CY = TY + 1, COR = CX * CY;
+    static constexpr size_t smem(int nc) {
+        return sizeof(CornerTables) + (size_t)COR * 2 * nc * sizeof(double) + (size_t)(COR + CX + CY) * sizeof(Dist);
+    }
+};
 
-template <int NC, bool TABLES>
+template <int NC, bool TABLES, int TY>
 __global__ void __launch_bounds__(kGenThreads)
     kernel_gen(Geometry g, GenOut o, unsigned comps, int n0, int n1, int per, void* __restrict__ out) {
-    constexpr int CX = kGenCX, NT = kGenThreads;
+    constexpr int CX = GenTile<TY>::CX, CY = GenTile<TY>::CY, COR = GenTile<TY>::COR, NT = kGenThreads;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     CornerTables& tab = *reinterpret_cast<CornerTables*>(smem_raw);
     double* F = reinterpret_cast<double*>(smem_raw + sizeof(CornerTables));  // corner terms of the level above
-    double* D = F + kGenCor * NC;   // level minus the level above
-    Dist* rxy = reinterpret_cast<Dist*>(D + kGenCor * NC);  // sqrt(x^2 + y^2) per corner
-    Dist* rxz = rxy + kGenCor;                              // sqrt(x^2 + z^2), sqrt(y^2 + z^2) of the level
+    double* D = F + COR * NC;   // level minus the level above
+    Dist* rxy = reinterpret_cast<Dist*>(D + COR * NC);  // sqrt(x^2 + y^2) per corner
+    Dist* rxz = rxy + COR;                              // sqrt(x^2 + z^2), sqrt(y^2 + z^2) of the level
     Dist* ryz = rxz + CX;
     const int tid = threadIdx.x, tx = tid % kGenTX, ty0 = tid / kGenTX;
-    const int u0 = blockIdx.x * kGenTX, v0 = blockIdx.y * kGenTY;
+    const int u0 = blockIdx.x * kGenTX, v0 = blockIdx.y * TY;
     const int u = u0 + tx;
     const int first = n0 + blockIdx.z * per, last = min(n1, first + per);
 
@@ -142,16 +143,16 @@ __global__ void __launch_bounds__(kGenThreads)
     auto cy_of = [&](int cy) { return (0.5 - (v0 + cy)) * g.dy; };
     if constexpr (TABLES) {
         for (int e = tid; e < CornerTables::LOGS; e += NT) corner_table_entry(tab, e);
-        for (int e = tid; e < kGenCor; e += NT) rxy[e] = distance(cx_of(e % CX), cy_of(e / CX));
+        for (int e = tid; e < COR; e += NT) rxy[e] = distance(cx_of(e % CX), cy_of(e / CX));
     }
     // corner terms of z-level z into F and, but for the first level, their change into D
     auto level = [&](double z, bool difference) {
         if constexpr (TABLES) {
             if (tid < CX) rxz[tid] = distance(cx_of(tid), z);
-            else if (tid >= 64 && tid < 64 + kGenCY) ryz[tid - 64] = distance(cy_of(tid - 64), z);
+            else if (tid >= 64 && tid < 64 + CY) ryz[tid - 64] = distance(cy_of(tid - 64), z);
         }
         __syncthreads();  // distances in place; D and the tables free or in place
-        for (int e = tid; e < kGenCor; e += NT) {
+        for (int e = tid; e < COR; e += NT) {
             const int cy = e / CX, cx = e - cy * CX;
             if (u0 + cx > g.nx || v0 + cy > g.ny) continue;
             double t[NC];
@@ -171,7 +172,7 @@ __global__ void __launch_bounds__(kGenThreads)
     level(-g.h - first * g.dz, false);
     for (int n = first; n < last; ++n) {
         level(-g.h - (n + 1) * g.dz, true);
-        for (int ty = ty0; ty < kGenTY; ty += NT / kGenTX) {
+        for (int ty = ty0; ty < TY; ty += NT / kGenTX) {
             const int v = v0 + ty;
             if (u >= g.nx || v >= g.ny) continue;
 #pragma unroll
@@ -214,20 +215,40 @@ __global__ void __launch_bounds__(kGenThreads)
     }
 }
 
-template <int NC, bool TABLES>
+// Tiles of TY rows, and the runs of layers that they are cut into: each run
+// costs one level more, so at least 8 layers, and no more runs than give every
+// SM 12 CTAs.
+dim3 gen_grid(const Geometry& g, int nz, int ty, int* per) {
+    dim3 grid((g.nx + kGenTX - 1) / kGenTX, (g.ny + ty - 1) / ty);
+    const int tiles = (int)(grid.x * grid.y);
+    const int want = std::max(1, std::min((12 * 152 + tiles - 1) / tiles, nz / 8));
+    *per = (nz + want - 1) / want;
+    grid.z = (nz + *per - 1) / *per;
+    return grid;
+}
+
+template <int NC, bool TABLES, int TY>
 cudaError_t gen_launch(const Geometry& g, const GenOut& o, unsigned comps, int n0, int n1, void* out, cudaStream_t s) {
-    constexpr auto k = kernel_gen<NC, TABLES>;
+    constexpr auto k = kernel_gen<NC, TABLES, TY>;
     cudaError_t e = ensure_smem_limit<k>();
     if (e != cudaSuccess) return e;
-    dim3 grid((g.nx + kGenTX - 1) / kGenTX, (g.ny + kGenTY - 1) / kGenTY);
-    // runs of layers: each costs one level more, so at least 8 layers, and no
-    // more runs than give every SM 12 CTAs
-    const int nz = n1 - n0, tiles = (int)(grid.x * grid.y);
-    const int want = std::max(1, std::min((12 * 152 + tiles - 1) / tiles, nz / 8));
-    const int per = (nz + want - 1) / want;
-    grid.z = (nz + per - 1) / per;
-    k<<<grid, kGenThreads, gen_smem(NC), s>>>(g, o, comps, n0, n1, per, out);
+    int per;
+    const dim3 grid = gen_grid(g, n1 - n0, TY, &per);
+    k<<<grid, kGenThreads, GenTile<TY>::smem(NC), s>>>(g, o, comps, n0, n1, per, out);
     return cudaGetLastError();
+}
+
+template <int NC>
+cudaError_t gen_either(const Geometry& g, const GenOut& o, unsigned comps, int n0, int n1, void* out, cudaStream_t s) {
+    if (o.tables) return gen_launch<NC, true, 16>(g, o, comps, n0, n1, out, s);
+    // the library functions' corners take long enough that a mesh of fewer
+    // tiles than SMs waits for the trips of one tile: two of 256 corners a level
+    // with 8 rows, three with 16 (16 x 16 x 4 FP64 plan, six components: 383 us
+    // with 8, 510 with 16; where the SMs are full 16 rows share more corners)
+    int per;
+    const dim3 grid = gen_grid(g, n1 - n0, 16, &per);
+    if (grid.x * grid.y * grid.z < 152) return gen_launch<NC, false, 8>(g, o, comps, n0, n1, out, s);
+    return gen_launch<NC, false, 16>(g, o, comps, n0, n1, out, s);
 }
 
 }  // namespace
@@ -235,10 +256,8 @@ cudaError_t gen_launch(const Geometry& g, const GenOut& o, unsigned comps, int n
 cudaError_t launch_kernel_gen(const Geometry& g, const GenOut& o, unsigned comps, int n0, int n1, void* out,
                               cudaStream_t s) {
     comps &= kCompBits;
-    const bool nine = comps & (GRAV_GX | GRAV_GY);
-    if (o.tables)
-        return nine ? gen_launch<9, true>(g, o, comps, n0, n1, out, s) : gen_launch<7, true>(g, o, comps, n0, n1, out, s);
-    return nine ? gen_launch<9, false>(g, o, comps, n0, n1, out, s) : gen_launch<7, false>(g, o, comps, n0, n1, out, s);
+    return comps & (GRAV_GX | GRAV_GY) ? gen_either<9>(g, o, comps, n0, n1, out, s)
+                                       : gen_either<7>(g, o, comps, n0, n1, out, s);
 }
 
 // The eight corner terms cancel, so a kernel value carries their rounding
