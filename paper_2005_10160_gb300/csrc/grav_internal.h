@@ -230,9 +230,9 @@ cudaError_t launch_row_c2r(int log_p, const void* in0, const void* in1, int I, i
 
 // FP32 rows of P = 2^log_p = 128 .. 2048 points with at most P / 2 nonzero
 // inputs or wanted outputs (row_groups.cu): arguments and layouts as the
-// launchers above; cudaErrorNotSupported when the sizes or alignments do not
-// fit (other lengths, l_in or l_out > P / 2, odd i_pad or batch stride, a
-// workspace that is not 16-byte aligned), and the caller takes another kernel.
+// launchers above.  Required, and true of every plan: l_in or l_out <= P / 2, an
+// even i_pad and batch stride, 16-byte aligned workspaces; anything else is
+// cudaErrorInvalidValue.
 cudaError_t launch_row_r2c_group(int log_p, const float* in, size_t in_ostride, size_t in_istride, int l_in, int I,
                                  int O, void* out, int i_pad, const void* tw, int log_t, cudaStream_t s, Batch b);
 cudaError_t launch_row_c2r_group(int log_p, const void* in0, const void* in1, int I, int O, int i_pad, float* out,
@@ -241,8 +241,8 @@ cudaError_t launch_row_c2r_group(int log_p, const void* in0, const void* in1, in
 // FP32 transforms of `rows` contiguous complex rows (the y passes of the
 // equal-dimension plans), row_groups.cu: forward, l_in <= P / 2 values
 // zero-padded to P = 2^log_p = 128 .. 2048; inverse, the first l_out <= P / 2
-// of P = 128 .. 2048 outputs kept.  Strides in complex elements;
-// cudaErrorNotSupported when the sizes or alignments do not fit.
+// of P = 128 .. 2048 outputs kept.  Strides in complex elements, even for the
+// forward's output, which is 16-byte aligned; cudaErrorInvalidValue otherwise.
 cudaError_t launch_rows_fwd_group(int log_p, const void* in, size_t in_stride, int l_in, void* out, size_t out_stride,
                                   long rows, const void* tw, int log_t, cudaStream_t s);
 cudaError_t launch_rows_inv_group(int log_p, const void* in, size_t in_stride, void* out, size_t out_stride, int l_out,

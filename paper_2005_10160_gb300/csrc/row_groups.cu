@@ -474,7 +474,7 @@ bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 
 cudaError_t launch_row_r2c_group(int log_p, const float* in, size_t in_ostride, size_t in_istride, int l_in, int I,
                                  int O, void* out, int i_pad, const void* tw, int log_t, cudaStream_t s, Batch b) {
     if (log_p < 7 || log_p > 11 || l_in > (1 << log_p) / 2 || i_pad % 2 || b.out % 2 || !aligned16(out))
-        return cudaErrorNotSupported;
+        return cudaErrorInvalidValue;
     switch (log_p) {
         case 7: return r2c_launch<64>(in, in_ostride, in_istride, l_in, I, O, out, i_pad, tw, log_t, s, b);
         case 8: return r2c_launch<128>(in, in_ostride, in_istride, l_in, I, O, out, i_pad, tw, log_t, s, b);
@@ -488,7 +488,7 @@ cudaError_t launch_row_c2r_group(int log_p, const void* in0, const void* in1, in
                                  size_t out_stride, int l_out, const void* tw, int log_t, cudaStream_t s, Batch b) {
     if (log_p < 7 || log_p > 11 || l_out > (1 << log_p) / 2 || i_pad % 2 || b.in % 2 || !aligned16(in0) ||
         !aligned16(in1))
-        return cudaErrorNotSupported;
+        return cudaErrorInvalidValue;
     switch (log_p) {
         case 7: return c2r_either<64>(in0, in1, I, O, i_pad, out, out_stride, l_out, tw, log_t, s, b);
         case 8: return c2r_either<128>(in0, in1, I, O, i_pad, out, out_stride, l_out, tw, log_t, s, b);
@@ -501,7 +501,7 @@ cudaError_t launch_row_c2r_group(int log_p, const void* in0, const void* in1, in
 cudaError_t launch_rows_fwd_group(int log_p, const void* in, size_t in_stride, int l_in, void* out, size_t out_stride,
                                   long rows, const void* tw, int log_t, cudaStream_t s) {
     if (log_p < 7 || log_p > 11 || l_in > (1 << log_p) / 2 || out_stride % 2 || !aligned16(out))
-        return cudaErrorNotSupported;
+        return cudaErrorInvalidValue;
     switch (log_p) {
         case 7: return rows_fwd_launch<64>(in, in_stride, l_in, out, out_stride, rows, tw, log_t, s);
         case 8: return rows_fwd_launch<128>(in, in_stride, l_in, out, out_stride, rows, tw, log_t, s);
@@ -513,7 +513,7 @@ cudaError_t launch_rows_fwd_group(int log_p, const void* in, size_t in_stride, i
 
 cudaError_t launch_rows_inv_group(int log_p, const void* in, size_t in_stride, void* out, size_t out_stride, int l_out,
                                   long rows, const void* tw, int log_t, cudaStream_t s) {
-    if (log_p < 7 || log_p > 11 || l_out > (1 << log_p) / 2) return cudaErrorNotSupported;
+    if (log_p < 7 || log_p > 11 || l_out > (1 << log_p) / 2) return cudaErrorInvalidValue;
     switch (log_p) {
         case 7: return rows_inv_launch<64>(in, in_stride, out, out_stride, l_out, rows, tw, log_t, s);
         case 8: return rows_inv_launch<128>(in, in_stride, out, out_stride, l_out, rows, tw, log_t, s);
