@@ -9,10 +9,11 @@ namespace grav {
 namespace {
 
 // Layer groups per CTA: one, except for 64-point columns, whose group is a
-// single warp: those take the layers in one go (up to 8 groups).  Measured at
-// 256 x 256 x 32 and 16 requests of 128 x 128 x 32, six components: one group
-// 49 and 112 us, two and four groups 51 and 152 us (the final sum over the
-// groups costs more than the shorter chain gains).  The rule looks at the plan
+// single warp: those take the layers in one go (up to 8 groups).  Measured in an
+// earlier form of the kernel, whole calls at 256 x 256 x 32 and 16 requests of
+// 128 x 128 x 32, six components (39 and 105 us now): one group 49 and 112 us,
+// two and four groups 51 and 152 us (the final sum over the groups costs more
+// than the shorter chain gains).  The rule looks at the plan
 // only: the order of the layer sum, and so the result, must not depend on how
 // many requests share a launch.
 template <int N> int layer_groups(const ColumnArgs& a) {

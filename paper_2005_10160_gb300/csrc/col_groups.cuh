@@ -8,13 +8,17 @@
 // accumulates eight layers, and only a barrier of the group (a warp sync for
 // N = 64) stands between.
 //
-// Forward: one CTA per (kx, ky parity) holds `groups` layer groups that take
-// the rounds in turn, each with its own compensated sums; at the end the
-// first group adds them up and runs the inverse transforms of all
-// components at once (one per transform slot, at most eight).  More groups
-// per CTA shorten the serial chain of a small problem; with enough CTAs to
-// fill the machine one group does.  The next round's rows are read into
-// registers before the accumulation, and the spectra one layer ahead.
+// Forward: one CTA per (kx, ky parity).  128- and 256-point columns run one
+// layer group, J threads, through all rounds; a 64-point group is a single warp,
+// so a CTA holds up to eight that take the rounds in turn, each with its own
+// compensated sums, which the first group adds up.  Then the inverse transforms
+// of all components run at once (one per transform slot, at most eight).  The
+// next round's rows are read into registers before the accumulation, and the
+// spectra one layer ahead.  The sum is plain over the eight layers of a round and
+// compensated over the rounds; compensated every four layers it is no closer to
+// 64 bits (1.8e-7 of the field at 256 x 256 x 32, 1.4e-7 for the requests below,
+// either way) and takes 41.4 against 39.1 and 116 against 105 us for the whole
+// calls.
 //
 // Adjoint: one CTA per kx and chunk of layers, both ky parities (N threads):
 // the residual columns of all components are transformed at once, each
@@ -24,12 +28,10 @@
 // through shared memory and added, so each layer's column is written once,
 // Z[kx][n][y] (ColumnArgs::z_summed).
 //
-// Bound by issue and latency, not by memory: at 256 x 256 x 32 with six
-// components (9.5 M warp instructions, 52 MB of spectra) the forward takes 24
-// us at 48% issue slots busy, 35 us as the block-FFT kernel it replaced; the
-// adjoint 25 us, 75 before.  16 requests of 128 x 128 x 32: forward 129 -> 71
-// us.  At three CTAs of 256 threads an SM (85 registers) the forward spills
-// and is slower (59.6 against 51.4 us for the whole forward).
+// Bound by latency, not by memory: under ncu (caches kept) at 256 x 256 x 32 with
+// six components (52 MB of spectra) the forward takes 25 us at 42% of the issue
+// slots, the block-FFT kernel it replaced 35; the adjoint 22 us at 40%, 75 before.
+// 16 requests of 128 x 128 x 32: forward 74 us at 46%, 129 before.
 #pragma once
 #include "async_copy.cuh"
 #include "grav_internal.h"
@@ -47,8 +49,9 @@ template <int N> struct ColGroup {
     // slots of one 16-lane phase start L complex values apart modulo 16
     static constexpr int AREA = (G::TR + 15) / 16 * 16 + G::L % 16;
     static constexpr int MAXG = 256 / J;  // layer groups of a forward CTA
-    // forward CTAs of six and more components keep their compensation terms
-    // in shared memory (in registers they spill at 128 a thread)
+    // forward CTAs of six and more components keep their compensation terms in
+    // shared memory, which leaves six without spills at 128 registers a thread;
+    // seven still spill 8 to 88 bytes and eight 196 to 244
     static constexpr bool cmp_in_smem(int nc) { return nc >= 6; }
     static constexpr size_t fwd_smem(int groups, int nc) {
         return (size_t)(N + groups * (SLOTS * AREA + (cmp_in_smem(nc) ? 2 * nc * J : 0))) * sizeof(float2);

@@ -112,8 +112,9 @@ __device__ __forceinline__ float2 split_pair(double v) {
 // above in shared memory, and every thread forms its offsets' kernel values
 // from four differences.  blockIdx.z takes a run of `per` layers.
 //
-// Bound by FP64 issue.  1024 x 1024 x 100, six components: 65 ms with the
-// tables, 92 ms with the library's asinh and atan and tiles of 32 x 8.
+// Bound by the FP64 pipe, 86% active with the tables (four layers of 1024 x
+// 1024).  1024 x 1024 x 100, six components: 65 ms with the tables, 92 ms with the library's
+// asinh and atan and tiles of 32 x 8.
 constexpr int kGenTX = 32, kGenThreads = 256;
 template <int TY> struct GenTile {
     static constexpr int CX = kGenTX + 1, CY = TY + 1, COR = CX * CY;
@@ -243,7 +244,7 @@ cudaError_t gen_either(const Geometry& g, const GenOut& o, unsigned comps, int n
     if (o.tables) return gen_launch<NC, true, 16>(g, o, comps, n0, n1, out, s);
     // the library functions' corners take long enough that a mesh of fewer
     // tiles than SMs waits for the trips of one tile: two of 256 corners a level
-    // with 8 rows, three with 16 (16 x 16 x 4 FP64 plan, six components: 383 us
+    // with 8 rows, three with 16 (16 x 16 x 4 FP64 plan, six components: 370 us
     // with 8, 510 with 16; where the SMs are full 16 rows share more corners)
     int per;
     const dim3 grid = gen_grid(g, n1 - n0, 16, &per);

@@ -1,7 +1,8 @@
 // Forward column stage for 1024-point FP32 column transforms (Py = 2048)
 // with one warp per layer transform.
 //
-// 16 warps at 128 registers a thread (the whole register file).  Warps 0-7
+// 16 warps at 128 registers a thread (the whole register file; six components
+// spill 32 bytes of stores and 44 of loads, eight 84 and 144).  Warps 0-7
 // accumulate: thread t owns the mirror pairs 2t and 2t + 1 for every component
 // (the layer sum of Eq. 20 in the Fourier domain), as two-wide FP32
 // operations over the two pairs.  Warps 8-15 transform: each layer's
