@@ -135,21 +135,29 @@ struct Scalars {
     int* status;
 };
 // alpha, the same value in every thread.  A vanished gradient ends the
-// recurrence: nothing moves any more.
-__device__ __forceinline__ double step_length(const Scalars& k) {
+// recurrence: nothing moves any more.  RECORD: one thread of the grid notes a
+// step without a length (a gradient, but (q, q) + lam (p, p) = 0) or with one
+// past R's range.
+template <typename R, bool RECORD> __device__ __forceinline__ double step_length(const Scalars& k) {
     __shared__ double alpha;
     if (threadIdx.x == 0) {
-        const double gamma = k.gamma->value;
-        alpha = gamma == 0.0 ? 0.0 : gamma / (k.qq->value + k.lam * k.pp->value);
+        const double gamma = k.gamma->value, curv = k.qq->value + k.lam * k.pp->value;
+        const double a = gamma == 0.0 ? 0.0 : gamma / curv;
+        alpha = a;
+        if (RECORD && blockIdx.x == 0 && gamma != 0.0 && !isfinite((R)a) && *k.status == kStepsDone) {
+            if (curv == 0.0) *k.status = kNoStepLength;
+            else if (isfinite(a)) *k.status = kStepLengthRange;
+        }
     }
     __syncthreads();
     return alpha;
 }
 
-// r = w d, wr = w r, (r, r)
+// r = w d, wr = w r, (r, r); clears the status
 template <typename R>
 __global__ void __launch_bounds__(kVecThreads) cgls_first_data(const R* __restrict__ d, const R* __restrict__ w, R* __restrict__ r,
-                                                               R* __restrict__ wr, size_t n, Making rr) {
+                                                               R* __restrict__ wr, size_t n, Making rr, int* status) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) *status = kStepsDone;
     Squares<R> s;
     for (size_t i = (size_t)blockIdx.x * kVecThreads + threadIdx.x; i < n; i += (size_t)gridDim.x * kVecThreads) {
         const R v = w[i] * d[i];
@@ -172,17 +180,11 @@ __global__ void __launch_bounds__(kVecThreads) cgls_weigh(const R* __restrict__ 
     put_dot(qq, s.get([&](auto f) { each_data(q, n, f); }));
 }
 
-// r -= alpha q, wr = w r, (r, r); records a step without a length (a gradient,
-// but (q, q) + lam (p, p) = 0) or with one past R's range
+// r -= alpha q, wr = w r, (r, r)
 template <typename R>
 __global__ void __launch_bounds__(kVecThreads) cgls_step_data(Scalars k, const R* __restrict__ w, const R* __restrict__ q, R* __restrict__ r,
                                                               R* __restrict__ wr, size_t n, Making rr) {
-    const double step = step_length(k);
-    const R alpha = (R)step;
-    if (blockIdx.x == 0 && threadIdx.x == 0 && *k.status == kStepsDone) {
-        if (k.gamma->value != 0.0 && k.qq->value + k.lam * k.pp->value == 0.0) *k.status = kNoStepLength;
-        else if (!isinf(step) && isinf(alpha)) *k.status = kStepLengthRange;
-    }
+    const R alpha = (R)step_length<R, true>(k);
     Squares<R> s;
     for (size_t i = (size_t)blockIdx.x * kVecThreads + threadIdx.x; i < n; i += (size_t)gridDim.x * kVecThreads) {
         const R v = r[i] - alpha * q[i];
@@ -232,7 +234,7 @@ __global__ void __launch_bounds__(kVecThreads) cgls_step_model(Scalars k, bool f
                                                                R* __restrict__ g, R* __restrict__ m, size_t plane, int nz,
                                                                Making ss, Making xx) {
     using P = Pack<R, VEC>;
-    const R alpha = (R)step_length(k), lam = (R)k.lam;
+    const R alpha = (R)step_length<R, false>(k), lam = (R)k.lam;
     Squares<R> s2, x2;
     GRAV_FOR_LAYERS
             const P pv = *reinterpret_cast<const P*>(p + base + i);
@@ -369,9 +371,8 @@ int run_start(grav_plan* plan, const R* d, const R* w, const R* wm, int iters, v
     const Loop<R> L(plan, iters, work);
     constexpr int V = 16 / sizeof(R);
     cudaError_t e = cudaMemsetAsync(L.pp, 0, L.k.dots() * sizeof(Dot), s);  // no block done yet
-    if (e == cudaSuccess) e = cudaMemsetAsync(L.status, 0, sizeof(int), s);
     if (e != cudaSuccess) return cuda_fail(e, "grav_cgls_start");
-    cgls_first_data<R><<<L.gd, kVecThreads, 0, s>>>(d, w, L.r, L.wr, L.k.nd, L.first(L.rr(0)));
+    cgls_first_data<R><<<L.gd, kVecThreads, 0, s>>>(d, w, L.r, L.wr, L.k.nd, L.first(L.rr(0)), L.status);
     const int rc = grav_adjoint(plan, L.wr, L.g, s);
     if (rc != GRAV_OK) return rc;
     if (L.vec) cgls_first_model<R, V><<<L.gm, kVecThreads, 0, s>>>(wm, L.g, L.p, L.t, L.k.plane, L.k.nz, L.first(L.ss(0)), L.second(L.pp));
